@@ -86,3 +86,26 @@ def test_limits_and_degenerate_cases():
     assert st == smat.SMAT_ERR_INVALID_ARG
     for M in (A64, A32, N64, N32):
         M.close()
+
+
+@pytest.mark.parametrize("n", [1, 3, 4095, 4097, 32767, 32769, 65539, 622592, 622595, 1400001])
+def test_vector_kernel_sizes(n):
+    """The vector kernel's launch shapes (one CTA, one cluster, registers over
+    the whole GPU, streaming) at their edges and with n % 4 != 0, on
+    tridiag(-1, 4, -1): eigenvalues in (2, 6), so a relative residual of
+    1e-12 bounds the relative error by 3e-12 (plus rounding)."""
+    i = np.arange(n)
+    cols = np.stack([i - 1, i, i + 1], 1)
+    ok = (cols >= 0) & (cols < n)
+    val = np.broadcast_to(np.array([-1.0, 4.0, -1.0]), (n, 3))[ok].copy()
+    rowptr = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    A = synth.CSR(n, n, rowptr, cols[ok].astype(np.int32), val)
+    x_true = synth.uniform(3, 5, n)
+    b = oracle.spmv_csr(n, A.rowptr, A.colidx, A.val, x_true, threads=8)
+    A64, A32 = handles(A, tune=False)
+    xd = torch.zeros(n, dtype=torch.float64, device=DEV)
+    info = smat.cg_mixed(A64, A32, torch.from_numpy(b).to(DEV), xd, rtol=1e-12)
+    assert info["converged"], info
+    err = np.linalg.norm(xd.cpu().numpy() - x_true) / np.linalg.norm(x_true)
+    assert err <= 4e-12, err
+    A64.close(), A32.close()
