@@ -155,3 +155,23 @@ def test_model_reloads_while_other_threads_tune():
         scale = oracle.spmv_csr(A.m, A.rowptr, A.colidx, np.abs(A.val), np.abs(x), threads=8)
         assert np.all(np.abs(y - ref) <= 1e-12 * scale + 1e-300), M.plan()["name"]
         M.close()
+
+
+@pytest.mark.parametrize("B", [1, 4, 29, 33, 2400])
+def test_gradient_at_tile_edges(B):
+    """CTAs of 32 samples in groups of four: one sample, a full group, a ragged
+    last group, one sample in the last CTA, many CTAs.  FP32 sums of at most
+    2400 terms: 1e-4 of the gradient's norm is far above their rounding."""
+    p = _params(6)
+    rng = np.random.default_rng(7)
+    X = rng.standard_normal((B, 12)).astype(np.float32)
+    T = rng.random((B, 8)).astype(np.float32)
+    T /= T.sum(1, keepdims=True)
+    pd, xd, td = (torch.from_numpy(a).to(DEV) for a in (p, X, T))
+    g, loss = torch.empty_like(pd), torch.empty(1, device=DEV)
+    work = torch.empty(smat.smat_mlp_work_floats(B), device=DEV)
+    assert smat.smat_mlp_loss_grad(pd.data_ptr(), xd.data_ptr(), td.data_ptr(), B, g.data_ptr(), loss.data_ptr(),
+                                   work.data_ptr(), _stream()) == 0
+    ref_loss, ref_g = oracle.mlp_loss_grad(p.astype(np.float64), X.astype(np.float64), T.astype(np.float64))
+    assert abs(loss.item() - ref_loss) <= 1e-5 * abs(ref_loss)
+    assert np.linalg.norm(g.cpu().numpy() - ref_g) <= 1e-4 * np.linalg.norm(ref_g)
