@@ -87,7 +87,7 @@ typedef enum {
   SMAT_V_CSR_VEC4 = 1,   /* 4 lanes per row, shuffle reduction              */
   SMAT_V_CSR_VEC8 = 2,   /* 8 lanes per row                                  */
   SMAT_V_CSR_VEC32 = 3,  /* one warp per row                                 */
-  SMAT_V_CSR_MERGE = 4,  /* merge-path split of rows + nonzeros              */
+  SMAT_V_CSR_MERGE = 4,  /* entries split evenly over warps, whatever the rows */
   SMAT_V_ELL = 5,        /* column-major ELL, 16-byte vector loads           */
   SMAT_V_DIA = 6,        /* diagonal-major DIA                               */
   SMAT_V_COO = 7,        /* COO with segmented reduction                     */
@@ -644,7 +644,7 @@ smat_status_t smat_cast_f64_to_bf16(const double *in, uint16_t *out, int64_t n, 
 /* ------------------------------------------------------------------------ */
 /* Allocation-free product (the paper has no counterpart to this entry point) */
 /* ------------------------------------------------------------------------ */
-/* y = alpha*A*x + beta*y by merge-path CSR for callers that cannot allocate
+/* y = alpha*A*x + beta*y by evenly split CSR for callers that cannot allocate
  * device memory: a solver whose memory manager owns every device byte, code
  * that must not synchronise the device the way cudaMalloc/cudaFree may, or a
  * host that forbids allocation once its time-critical loop runs.  No handle
@@ -654,12 +654,11 @@ smat_status_t smat_cast_f64_to_bf16(const double *in, uint16_t *out, int64_t n, 
  * (FP64 for SMAT_F64, FP32 otherwise).  The input must be canonical CSR; it is
  * not validated.  alpha == 0 gives y = beta*y (0 when beta == 0) without
  * reading A or x, and beta == 0 makes y write-only, as in smat_spmv.
- * The kernels' only scratch, one carry and one merge-path coordinate per
- * tile of 2048 merge items, lives in a fixed 1.25 MiB array in the library's
- * device memory, held by every GPU that loads the library until the process
- * exits.  Limit: ceil((m + nnz) /
- * 2048) <= 65536, i.e. m + nnz <= 134,217,728; larger inputs return
- * SMAT_ERR_UNSUPPORTED without launching anything.  The first call on each
+ * The kernels' only scratch, one carry and one first row per tile of 256 to
+ * 2048 entries, lives in a fixed 1 MiB array in the library's device memory,
+ * held by every GPU that loads the library until the process exits.  Limit:
+ * m + nnz <= 134,217,728; larger inputs return SMAT_ERR_UNSUPPORTED without
+ * launching anything.  Arrays that start on 32 bytes are read fastest.  The first call on each
  * device looks up the array's address (cudaGetSymbolAddress) and keeps it for
  * the rest of the process; make that first call before any stream capture,
  * and do not call this entry point again after a cudaDeviceReset of a device

@@ -822,7 +822,7 @@ smat_status_t ensure_scratch(smat_s *h, int variant) {
 
 bool variant_ready(const smat_s *h, int v) {
   int fmt = variant_format(v);
-  if (v == SMAT_V_CSR_MERGE && h->m > 0 && !h->merge_coords) return false;
+  if (v == SMAT_V_CSR_MERGE && h->m > 0 && !h->flat_row) return false;
   if (fmt == SMAT_FMT_ELL && !h->ell_val) return false;
   if (fmt == SMAT_FMT_DIA && !h->dia_val) return false;
   if (fmt == SMAT_FMT_COO && !h->coo_row && !(h->nnz == 0)) return false;
@@ -841,11 +841,19 @@ smat_status_t prepare_variant(smat_s *h, int v, cudaStream_t s) {
   if (fmt != SMAT_FMT_CSR && !h->have_features) TRYS(compute_features(h, s));
   TRYS(build_format(h, fmt, s));
   TRYS(ensure_scratch(h, v));
-  if (v == SMAT_V_CSR_MERGE && !h->merge_coords && h->m > 0) {
+  if (v == SMAT_V_CSR_MERGE && !h->flat_row && h->m > 0) {
     void *p = nullptr;
-    TRY(dev_alloc(&p, (size_t)(merge_tiles(h->m, h->nnz) + 1) * 8));
-    h->merge_coords = p;
-    TRY(launch_merge_partition(h->rowptr, h->m, h->nnz, h->merge_coords, s));
+    DevBuf gaps(s);
+    int found = 0;
+    TRY(gaps.alloc(sizeof(int)));
+    TRY(cudaMemsetAsync(gaps.p, 0, sizeof(int), s));
+    TRY(dev_alloc(&p, (size_t)(flat_tiles(h->nnz) + 1) * 4));
+    cudaError_t e = launch_flat_rows(h, (int32_t *)p, gaps.as<int>(), s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&found, gaps.p, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) { dev_free(p); return st_of(e); }
+    h->flat_row = (int32_t *)p;
+    h->flat_gaps = found != 0;
   }
   return SMAT_OK;
 }
@@ -1182,7 +1190,7 @@ smat_status_t smat_destroy(smat_handle_t h) {
   dev_free(h->rowptr); dev_free(h->colidx); dev_free(h->val);
   free_format(h, SMAT_FMT_ELL); free_format(h, SMAT_FMT_DIA); free_format(h, SMAT_FMT_COO);
   free_ext_layouts(h);
-  dev_free(h->carry); dev_free(h->stage_x); dev_free(h->stage_y); dev_free(h->merge_coords);
+  dev_free(h->carry); dev_free(h->stage_x); dev_free(h->stage_y); dev_free(h->flat_row);
   if (h->pst[0]) {
     for (cudaStream_t st : h->pst) cudaStreamSynchronize(st);
     for (int q = 0; q < 2; ++q) {

@@ -125,9 +125,11 @@ struct smat_s {
   bool ext_known[4] = {false, false, false, false};
   double ext_slots[4] = {0, 0, 0, 0}, ext_bytes[4] = {0, 0, 0, 0};
 
-  // merge-path tile coordinates (int2 per tile boundary), computed once
-  void *merge_coords = nullptr;
-  // scratch for merge-path and COO carries
+  // SMAT_V_CSR_MERGE: the row of every tile's first entry, computed once, and
+  // whether a tile has so many (empty) rows that a pass of its own writes them
+  int32_t *flat_row = nullptr;
+  bool flat_gaps = false;
+  // scratch for CSR-merge and COO carries
   void *carry = nullptr;
   size_t carry_bytes = 0;
   // The buffers above serve the first stream that runs products on the
@@ -210,11 +212,6 @@ cudaError_t launch_bcsr_uniform(const smat_s *h, long long c, int *flag, cudaStr
 cudaError_t launch_spmv_ext(const smat_s *h, int variant, const void *alpha, const void *x,
                             const void *beta, void *y, cudaStream_t s);
 
-// Merge-path tiles of an m x ? matrix with nnz entries, and the kernel that
-// writes their (ntiles + 1) boundary coordinates (int2) to `coords`.
-long long merge_tiles(long long m, long long nnz);
-cudaError_t launch_merge_partition(const int32_t *rowptr, long long m, long long nnz, void *coords,
-                                   cudaStream_t s);
 // Per-product scratch: carries (merge-path, COO, HYB and SPLIT tails) and
 // SPLIT's chunk sums.
 struct Scratch {
@@ -227,6 +224,14 @@ struct Scratch {
 // uses the handle's buffers without making s their owner.
 cudaError_t stream_scratch(const smat_s *h, cudaStream_t s, Scratch *out, bool claim = true);
 void free_stream_scratch(smat_s *h);
+// CSR split evenly by entries (csr_flat.cu): its tiles, the kernels that fill
+// tile_row[tiles + 1] and set *gaps (zeroed by the caller), and the product.
+long long flat_tiles(long long nnz);
+cudaError_t launch_flat_rows(const smat_s *h, int32_t *tile_row, int *gaps, cudaStream_t s);
+cudaError_t launch_csr_flat(const smat_s *h, const Scratch &sc, const void *alpha, const void *x, const void *beta,
+                            void *y, cudaStream_t s);
+// y = beta*y (0 when beta == 0) on m rows; beta is a host scalar of the compute type.
+cudaError_t launch_beta_only(smat_dtype_t dtype, long long m, const void *beta, void *y, cudaStream_t s);
 // Size in bytes of the carry scratch a variant needs (0 if none).
 size_t carry_bytes_needed(const smat_s *h, int variant);
 // Kernel launches one product through `variant` issues.

@@ -26,11 +26,10 @@
 
 #include "smat_internal.h"
 #include "spmv_device.cuh"
+#include "warp_tile.cuh"
 
 namespace smat {
 namespace {
-
-constexpr unsigned FULL = 0xffffffffu;
 
 // ---------------------------------------------------------------------------
 // K7: CSR-scalar, one thread per row.
@@ -205,191 +204,6 @@ __device__ __forceinline__ T tile_carries(bool h, T c, T *open) {
     *open = o;
   }
   return in;
-}
-
-// Merge-path coordinate: number of row ends a among the first d merge items
-// of (rowptr[1..m]) and (0..nnz-1), row ends first on ties.
-__device__ __forceinline__ void merge_search(const int32_t *__restrict__ rowptr, long long m, long long nnz,
-                                             long long d, long long *a, long long *b) {
-  long long lo = d - nnz > 0 ? d - nnz : 0, hi = d < m ? d : m;
-  while (lo < hi) {
-    long long mid = (lo + hi) >> 1;
-    if ((long long)__ldg(rowptr + mid + 1) <= d - mid - 1) lo = mid + 1; else hi = mid;
-  }
-  *a = lo;
-  *b = d - lo;
-}
-
-// s_v[j] = val[b0 + j], s_x[j] = x[col[b0 + j]] for j < cnt: IPT coalesced
-// items per thread, every index and value load issued before the gathers.
-// Merge-path coordinates (a, b) of every tile boundary d = t*tile, t = 0..ntiles
-// (the last one clamped to m + nnz): one thread per boundary.
-__global__ void merge_partition_kernel(const int32_t *__restrict__ rowptr, long long m, long long nnz, long long tile,
-                                       long long ntiles, int2 *__restrict__ coords) {
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t <= ntiles;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long d = t * tile < m + nnz ? t * tile : m + nnz;
-    long long a, b;
-    merge_search(rowptr, m, nnz, d, &a, &b);
-    coords[t] = make_int2((int)a, (int)b);
-  }
-}
-
-template <typename V, typename T, int NT, int IPT>
-__device__ __forceinline__ void stage_pairs(const int32_t *__restrict__ col, const V *__restrict__ val,
-                                            const T *__restrict__ x, long long b0, int cnt, T *s_v, T *s_x) {
-  int c[IPT];
-  T v[IPT], xv[IPT];
-#pragma unroll
-  for (int q = 0; q < IPT; ++q) {
-    const int j = threadIdx.x + q * NT;
-    c[q] = j < cnt ? ld_idx(col + b0 + j) : 0;
-    v[q] = j < cnt ? (T)ld_val(val + b0 + j) : (T)0;
-  }
-#pragma unroll
-  for (int q = 0; q < IPT; ++q) xv[q] = (threadIdx.x + q * NT) < cnt ? __ldg(x + c[q]) : (T)0;
-#pragma unroll
-  for (int q = 0; q < IPT; ++q) {
-    const int j = threadIdx.x + q * NT;
-    if (j < cnt) {
-      s_v[j] = v[q];
-      s_x[j] = xv[q];
-    }
-  }
-}
-
-template <typename V, typename T, int NT, int IPT, int MODE>
-__global__ void __launch_bounds__(NT) csr_merge_kernel(const int32_t *__restrict__ rowptr,
-                                                       const int32_t *__restrict__ col,
-                                                       const V *__restrict__ val, const T *__restrict__ x,
-                                                       Epi<T, MODE> ep, T *__restrict__ y, long long m,
-                                                       long long nnz, const int2 *__restrict__ coords,
-                                                       int32_t *carry_row, T *carry_val) {
-  griddep_wait();
-  constexpr int TILE = NT * IPT;
-  __shared__ int32_t s_rowend[TILE + 1];
-  __shared__ T s_v[TILE], s_x[TILE];
-  const long long total = m + nnz;
-  const long long d0 = (long long)blockIdx.x * TILE;
-  const long long d1 = d0 + TILE < total ? d0 + TILE : total;
-  // the tile's merge-path coordinates, computed once per matrix
-  const int2 c0 = __ldg(coords + blockIdx.x), c1 = __ldg(coords + blockIdx.x + 1);
-  const long long a0 = c0.x, b0 = c0.y, a1 = c1.x, b1 = c1.y;
-  const int nrows = (int)(a1 - a0), nnzs = (int)(b1 - b0);
-  for (int i = threadIdx.x; i < nrows; i += NT) s_rowend[i] = __ldg(rowptr + a0 + 1 + i);
-  stage_pairs<V, T, NT, IPT>(col, val, x, b0, nnzs, s_v, s_x);
-  __syncthreads();
-  // this thread's start on the tile's merge path
-  const int items = (int)(d1 - d0);
-  const int dt = min((int)threadIdx.x * IPT, items);
-  int lo = dt - nnzs > 0 ? dt - nnzs : 0, hi = dt < nrows ? dt : nrows;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if ((long long)s_rowend[mid] <= b0 + (dt - mid - 1)) lo = mid + 1; else hi = mid;
-  }
-  int a = lo;
-  long long b = b0 + (dt - lo);
-  const int dend = min(dt + IPT, items);
-  T acc = 0, first_acc = 0;
-  int first_row = -1;
-  for (int it = dt; it < dend; ++it) {
-    if (a < nrows && (long long)s_rowend[a] <= b) {
-      if (first_row < 0) {
-        first_row = a;
-        first_acc = acc;
-      } else {
-        long long r = a0 + a;
-        y[r] = ep(acc, y, r);
-      }
-      acc = 0;
-      ++a;
-    } else {
-      acc = fused(acc, s_v[b - b0], s_x[b - b0]);
-      ++b;
-    }
-  }
-  T tile_open = 0;
-  const T incoming = tile_carries<T, NT>(first_row >= 0, acc, &tile_open);
-  if (first_row >= 0) {
-    long long r = a0 + first_row;
-    y[r] = ep(incoming + first_acc, y, r);
-  }
-  if (threadIdx.x == NT - 1) {
-    bool open = a1 < m && b1 > b0;
-    carry_row[blockIdx.x] = open ? (int32_t)a1 : -1;
-    carry_val[blockIdx.x] = open ? tile_open : (T)0;
-  }
-}
-
-// 32-byte streaming loads (sm_100 and later): one L1 request per 32-byte
-// sector.  Two 16-byte loads of one sector by the same thread are two
-// requests, and on a kernel bound by the rate of sector requests the second
-// one costs as much as the first (and comes back from L2 when the streamed
-// line was evicted in between).  p must be 32-byte aligned.
-__device__ __forceinline__ void ld32_i32(const int32_t *p, int *o) {
-  asm("ld.global.cs.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]), "=r"(o[4]), "=r"(o[5]), "=r"(o[6]), "=r"(o[7])
-      : "l"(p));
-}
-__device__ __forceinline__ void ld32_f32(const float *p, float *o) {
-  asm("ld.global.cs.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]), "=f"(o[4]), "=f"(o[5]), "=f"(o[6]), "=f"(o[7])
-      : "l"(p));
-}
-__device__ __forceinline__ void ld32_f64(const double *p, double *o) {
-  asm("ld.global.cs.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(o[0]), "=d"(o[1]), "=d"(o[2]), "=d"(o[3]) : "l"(p));
-}
-__device__ __forceinline__ bool aligned32(const void *p) { return ((uintptr_t)p & 31u) == 0; }
-
-// IPT consecutive int32 from p (16-byte aligned when `full`; 32-byte loads
-// when 32-byte aligned, uniform over a tile since runs start at multiples of 8).
-template <int IPT>
-__device__ __forceinline__ void load_i32_run(const int32_t *__restrict__ p, bool full, int valid, int (&o)[IPT],
-                                             int fill) {
-  if (full && IPT % 8 == 0 && aligned32(p)) {
-#pragma unroll
-    for (int q = 0; q < IPT / 8; ++q) ld32_i32(p + 8 * q, o + 8 * q);
-  } else if (full) {
-#pragma unroll
-    for (int q = 0; q < IPT / 4; ++q) {
-      int4 v = __ldcs(reinterpret_cast<const int4 *>(p) + q);
-      o[4 * q] = v.x; o[4 * q + 1] = v.y; o[4 * q + 2] = v.z; o[4 * q + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < IPT; ++q) o[q] = q < valid ? ld_idx(p + q) : fill;
-  }
-}
-
-template <typename V, int IPT>
-__device__ __forceinline__ void load_val_run(const V *__restrict__ p, bool full, int valid,
-                                             typename Compute<V>::T (&o)[IPT]) {
-  constexpr int R = 16 / (int)sizeof(V);
-  if constexpr (sizeof(V) == 8 && IPT % 4 == 0) {
-    if (full && aligned32(p)) {
-#pragma unroll
-      for (int q = 0; q < IPT / 4; ++q) ld32_f64(reinterpret_cast<const double *>(p) + 4 * q, o + 4 * q);
-      return;
-    }
-  } else if constexpr (sizeof(V) == 4 && IPT % 8 == 0) {
-    if (full && aligned32(p)) {
-#pragma unroll
-      for (int q = 0; q < IPT / 8; ++q) ld32_f32(reinterpret_cast<const float *>(p) + 8 * q, o + 8 * q);
-      return;
-    }
-  }
-  if (full) {
-#pragma unroll
-    for (int q = 0; q < IPT / R; ++q) {
-      typename Compute<V>::T t[R];
-      load_vals<V, R>(p + q * R, t);
-#pragma unroll
-      for (int r = 0; r < R; ++r) o[q * R + r] = t[r];
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < IPT; ++q) o[q] = q < valid ? (typename Compute<V>::T)ld_val(p + q) : 0;
-  }
 }
 
 // One chunk of up to IPT consecutive stored entries of a COO tile: each
@@ -590,31 +404,6 @@ __device__ __forceinline__ void split_chunk(long long c, const int32_t *__restri
 // blocks [nc, nc + tiles) are COO tiles of the short rows (the two sets
 // write disjoint rows).  One launch instead of two keeps the GPU full across
 // what was the boundary between them.
-// Within one warp whose 32 lanes' chunks form a tile: the inclusive
-// segmented sum of the lanes' open partial sums c, segments starting at the
-// lanes where a row ended (their c opens the next row).  A lane with a row
-// end gets the sum at the lane before it: the partials of the row its first
-// row end closes.  *open is the sum at lane 31, the row left open at the
-// tile's end.  Shuffles only; fixed order.
-template <typename T>
-__device__ __forceinline__ T warp_carries(bool h, T c, T *open) {
-  const int lane = threadIdx.x & 31;
-  int f = h ? 1 : 0;
-  T v = c;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const T vu = __shfl_up_sync(FULL, v, o);
-    const int fu = __shfl_up_sync(FULL, f, o);
-    if (lane >= o) {
-      if (!f) v = vu + v;
-      f |= fu;
-    }
-  }
-  *open = __shfl_sync(FULL, v, 31);
-  const T prev = __shfl_up_sync(FULL, v, 1);
-  return lane == 0 ? (T)0 : prev;
-}
-
 // A COO tile of one warp: lane l owns the 8 stored entries at b0 + 8 l; rows
 // ending inside a lane's entries are written as in the block tiles, the
 // first one after the warp's carries, and the row open at the tile's end is
@@ -811,7 +600,6 @@ int grid_for(long long work, int block, int max_blocks) {
   return (int)g;
 }
 
-constexpr int MERGE_NT = 256, MERGE_IPT = 8;
 // A COO product over (row, col, val) of length nnz, then the carry fix-up.
 template <typename V, typename T, int MODE>
 cudaError_t launch_coo(const Scratch &sc, const int32_t *row, const int32_t *col, const V *val, const T *x,
@@ -914,17 +702,6 @@ cudaError_t spmv_mode(const smat_s *h, const Scratch &sc, int variant, typename 
     case SMAT_V_CSR_VEC32:
       (void)launch_pdl(csr_vector_kernel<V, T, 32, MODE>, dim3(grid_for(m * 32, 256, 1 << 20)), dim3(256), 0, s, h->rowptr, h->colidx, val, x, ep, y, m);
       break;
-    case SMAT_V_CSR_MERGE: {
-      long long tiles = (m + h->nnz + MERGE_NT * MERGE_IPT - 1) / (MERGE_NT * MERGE_IPT);
-      int32_t *crow = (int32_t *)sc.carry;
-      T *cval = (T *)((char *)sc.carry + ((tiles * 4 + 15) / 16) * 16);
-      (void)launch_pdl(csr_merge_kernel<V, T, MERGE_NT, MERGE_IPT, MODE>, dim3((unsigned)tiles), dim3(MERGE_NT), 0, s,
-          h->rowptr, h->colidx, val, x, ep, y, m, h->nnz, (const int2 *)h->merge_coords, crow, cval);
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-      if (tiles > 1)
-        (void)launch_pdl(carry_fixup_kernel<T, MODE>, dim3(grid_for(tiles, 256, 152 * 8)), dim3(256), 0, s, crow, cval, tiles, ep, y);
-    } break;
     case SMAT_V_ELL:
       launch_ell_dia<V, MODE, false>(h, x, ep, y, s, u_req, lane_req);
       break;
@@ -997,18 +774,9 @@ cudaError_t spmv_typed(const smat_s *h, const Scratch &sc, int variant, const vo
 
 }  // namespace
 
-long long merge_tiles(long long m, long long nnz) { return (m + nnz + MERGE_NT * MERGE_IPT - 1) / (MERGE_NT * MERGE_IPT); }
-
-cudaError_t launch_merge_partition(const int32_t *rowptr, long long m, long long nnz, void *coords, cudaStream_t s) {
-  const long long tiles = merge_tiles(m, nnz);
-  merge_partition_kernel<<<grid_for(tiles + 1, 256, 152 * 8), 256, 0, s>>>(rowptr, m, nnz, MERGE_NT * MERGE_IPT,
-                                                                          tiles, (int2 *)coords);
-  return cudaGetLastError();
-}
-
 size_t carry_bytes_needed(const smat_s *h, int variant) {
   long long tiles = 0;
-  if (variant == SMAT_V_CSR_MERGE) tiles = (h->m + h->nnz + MERGE_NT * MERGE_IPT - 1) / (MERGE_NT * MERGE_IPT);
+  if (variant == SMAT_V_CSR_MERGE) tiles = flat_tiles(h->nnz);
   else if (variant == SMAT_V_COO) tiles = (h->nnz + COO_TILE - 1) / COO_TILE;
   else if (variant == SMAT_V_HYB) tiles = (h->hyb_ncoo + COO_TILE - 1) / COO_TILE;
   else if (variant == SMAT_V_SPLIT) tiles = (h->split_ns + SPLIT_TILE - 1) / SPLIT_TILE;
@@ -1020,8 +788,8 @@ size_t carry_bytes_needed(const smat_s *h, int variant) {
 int spmv_launch_count(const smat_s *h, int variant) {
   if (h->m == 0) return 0;
   if (variant == SMAT_V_CSR_MERGE) {
-    long long tiles = (h->m + h->nnz + MERGE_NT * MERGE_IPT - 1) / (MERGE_NT * MERGE_IPT);
-    return 1 + (tiles > 1);
+    const long long tiles = flat_tiles(h->nnz);
+    return (h->flat_gaps || h->nnz == 0) + (tiles > 0) + (tiles > 1);
   }
   if (variant == SMAT_V_COO) {
     long long tiles = (h->nnz + COO_TILE - 1) / COO_TILE;
@@ -1051,18 +819,22 @@ __global__ void beta_only_kernel(T *__restrict__ y, long long m, T beta) {
 }
 
 template <typename T>
-cudaError_t beta_only(const smat_s *h, const void *beta_p, void *y, cudaStream_t s) {
+cudaError_t beta_only(long long m, const void *beta_p, void *y, cudaStream_t s) {
   const T beta = *(const T *)beta_p;
-  if (h->m == 0) return cudaSuccess;
-  if (beta == (T)0) return cudaMemsetAsync(y, 0, (size_t)h->m * sizeof(T), s);
-  (void)launch_pdl(beta_only_kernel<T>, dim3(grid_for(h->m, 256, 152 * 8)), dim3(256), 0, s, (T *)y, h->m, beta);
+  if (m == 0) return cudaSuccess;
+  if (beta == (T)0) return cudaMemsetAsync(y, 0, (size_t)m * sizeof(T), s);
+  (void)launch_pdl(beta_only_kernel<T>, dim3(grid_for(m, 256, 152 * 8)), dim3(256), 0, s, (T *)y, m, beta);
   return cudaGetLastError();
+}
+
+cudaError_t launch_beta_only(smat_dtype_t dtype, long long m, const void *beta, void *y, cudaStream_t s) {
+  return dtype == SMAT_F64 ? beta_only<double>(m, beta, y, s) : beta_only<float>(m, beta, y, s);
 }
 
 cudaError_t launch_spmv(const smat_s *h, int variant, const void *alpha, const void *x, const void *beta,
                         void *y, cudaStream_t s, bool claim) {
   if (h->dtype == SMAT_F64 ? *(const double *)alpha == 0.0 : *(const float *)alpha == 0.0f)
-    return h->dtype == SMAT_F64 ? beta_only<double>(h, beta, y, s) : beta_only<float>(h, beta, y, s);
+    return launch_beta_only(h->dtype, h->m, beta, y, s);
   // ELL, DIA and HYB read x and write y, and BCSR reads x, with vector
   // accesses of up to 16 bytes; vectors that are not 16-byte aligned take the
   // CSR-scalar kernel instead.
@@ -1075,6 +847,7 @@ cudaError_t launch_spmv(const smat_s *h, int variant, const void *alpha, const v
     cudaError_t e = stream_scratch(h, s, &sc, claim);
     if (e != cudaSuccess) return e;
   }
+  if (variant == SMAT_V_CSR_MERGE) return h->m > 0 ? launch_csr_flat(h, sc, alpha, x, beta, y, s) : cudaSuccess;
   switch (h->dtype) {
     case SMAT_F64: return spmv_typed<double>(h, sc, variant, alpha, x, beta, y, s, 0, -1);
     case SMAT_F32: return spmv_typed<float>(h, sc, variant, alpha, x, beta, y, s, 0, -1);
@@ -1101,129 +874,3 @@ cudaError_t launch_spmv_width(const smat_s *h, int variant, int u, int lane, con
 }
 
 }  // namespace smat
-
-// ---------------------------------------------------------------------------
-// Merge-path CSR SpMV that allocates nothing.
-//
-// Some callers cannot call cudaMalloc: a solver that runs under a memory
-// manager owning every device byte, code that must not synchronise the device
-// (cudaMalloc/cudaFree may), or a host whose allocation calls are forbidden
-// once its time-critical loop has started.  For them this entry point keeps
-// the only scratch the kernel needs -- one carry (row, partial sum) per tile
-// -- in a fixed array in the library's own device memory.  Every GPU that
-// loads the library holds that array (1.25 MiB) until the process exits.
-// The array's address is looked up once per device, on the first call made
-// with that device current; make that first call before any stream capture.
-// All calls share the array, so calls whose kernels overlap on the GPU race:
-// order them on one stream, or synchronise between them.  Nothing in the
-// array has to start at zero: each call writes every carry and tile
-// coordinate it later reads.
-// ---------------------------------------------------------------------------
-#include <mutex>
-
-namespace smat {
-namespace {
-
-// The array holds three regions, for at most 65,536 tiles of 2048 merge items:
-constexpr long long NOALLOC_MAX_TILES = 65536;
-// [0, 256 KiB): each tile's carry row, int32
-constexpr size_t NOALLOC_ROW_BYTES = NOALLOC_MAX_TILES * 4;
-// [256 KiB, 768 KiB): each tile's carry value, 8 bytes (FP64) or 4 (FP32)
-constexpr size_t NOALLOC_VAL_BYTES = NOALLOC_MAX_TILES * 8;
-// [768 KiB, 1.25 MiB + 8 B): the merge-path coordinate (row, entry) of each
-// of the tiles + 1 tile boundaries, int2
-constexpr size_t NOALLOC_COORD_OFFSET = NOALLOC_ROW_BYTES + NOALLOC_VAL_BYTES;
-constexpr size_t NOALLOC_BYTES = NOALLOC_COORD_OFFSET + (NOALLOC_MAX_TILES + 1) * 8;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
-
-constexpr int NOALLOC_MAX_DEVICES = 64;
-std::mutex g_noalloc_mu;
-void *g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
-
-// Device address of the scratch array for the current device, looked up on
-// the first call with that device current and kept for the process's life:
-// after cudaDeviceReset the kept address is stale, so this entry point must
-// not be called again in a process that has reset a device it used.
-cudaError_t noalloc_scratch(void **out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= NOALLOC_MAX_DEVICES) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lock(g_noalloc_mu);
-  if (!g_noalloc_ptr[dev]) {
-    void *p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-    if (e != cudaSuccess) return e;
-    g_noalloc_ptr[dev] = p;
-  }
-  *out = g_noalloc_ptr[dev];
-  return cudaSuccess;
-}
-
-template <typename V, int MODE>
-cudaError_t merge_noalloc_mode(long long m, long long nnz, const int32_t *rowptr, const int32_t *colidx,
-                               const void *vals, typename Compute<V>::T alpha, const void *x_p,
-                               typename Compute<V>::T beta, void *y_p, unsigned char *scratch, cudaStream_t s) {
-  typedef typename Compute<V>::T T;
-  const Epi<T, MODE> ep{alpha, beta};
-  const long long tiles = (m + nnz + MERGE_NT * MERGE_IPT - 1) / (MERGE_NT * MERGE_IPT);
-  int32_t *crow = (int32_t *)scratch;
-  T *cval = (T *)(scratch + NOALLOC_ROW_BYTES);
-  int2 *coords = (int2 *)(scratch + NOALLOC_COORD_OFFSET);
-  cudaError_t e = launch_merge_partition(rowptr, m, nnz, coords, s);
-  if (e != cudaSuccess) return e;
-  csr_merge_kernel<V, T, MERGE_NT, MERGE_IPT, MODE><<<(unsigned)tiles, MERGE_NT, 0, s>>>(
-      rowptr, colidx, (const V *)vals, (const T *)x_p, ep, (T *)y_p, m, nnz, coords, crow, cval);
-  e = cudaGetLastError();
-  if (e != cudaSuccess || tiles <= 1) return e;
-  carry_fixup_kernel<T, MODE><<<grid_for(tiles, 256, 152 * 8), 256, 0, s>>>(crow, cval, tiles, ep, (T *)y_p);
-  return cudaGetLastError();
-}
-
-template <typename V>
-cudaError_t merge_noalloc_typed(long long m, long long nnz, const int32_t *rowptr, const int32_t *colidx,
-                                const void *vals, const void *alpha_p, const void *x_p, const void *beta_p,
-                                void *y_p, unsigned char *scratch, cudaStream_t s) {
-  typedef typename Compute<V>::T T;
-  const T alpha = *(const T *)alpha_p, beta = *(const T *)beta_p;
-  // alpha == 0: y = beta*y (0 when beta == 0), reading neither A nor x, as in
-  // smat_spmv, so that non-finite values in x cannot reach y
-  if (alpha == (T)0) {
-    if (beta == (T)0) return cudaMemsetAsync(y_p, 0, (size_t)m * sizeof(T), s);
-    beta_only_kernel<T><<<grid_for(m, 256, 152 * 8), 256, 0, s>>>((T *)y_p, m, beta);
-    return cudaGetLastError();
-  }
-  switch (epi_mode((double)alpha, (double)beta)) {
-    case EPI_COPY: return merge_noalloc_mode<V, EPI_COPY>(m, nnz, rowptr, colidx, vals, alpha, x_p, beta, y_p, scratch, s);
-    case EPI_SCALE: return merge_noalloc_mode<V, EPI_SCALE>(m, nnz, rowptr, colidx, vals, alpha, x_p, beta, y_p, scratch, s);
-    default: return merge_noalloc_mode<V, EPI_AXPBY>(m, nnz, rowptr, colidx, vals, alpha, x_p, beta, y_p, scratch, s);
-  }
-}
-
-}  // namespace
-}  // namespace smat
-
-extern "C" smat_status_t smat_spmv_csr_merge_noalloc(int64_t m, int64_t n, int64_t nnz, const int32_t *rowptr,
-                                                     const int32_t *colidx, const void *vals, smat_dtype_t dtype,
-                                                     const void *alpha, const void *x, const void *beta, void *y,
-                                                     void *stream) {
-  using namespace smat;
-  if (m < 0 || n < 0 || nnz < 0 || !alpha || !beta) return SMAT_ERR_INVALID_ARG;
-  if (dtype != SMAT_F64 && dtype != SMAT_F32 && dtype != SMAT_BF16) return SMAT_ERR_INVALID_ARG;
-  if (m == 0) return SMAT_OK;
-  if (!rowptr || !y || (nnz > 0 && (!colidx || !vals || !x))) return SMAT_ERR_INVALID_ARG;
-  if (m > INT32_MAX - 1 || n > INT32_MAX || nnz > INT32_MAX) return SMAT_ERR_UNSUPPORTED;
-  const long long tiles = (m + nnz + MERGE_NT * MERGE_IPT - 1) / (MERGE_NT * MERGE_IPT);
-  if (tiles > NOALLOC_MAX_TILES) return SMAT_ERR_UNSUPPORTED;  // beyond the fixed scratch
-  void *scratch = nullptr;
-  cudaError_t e = noalloc_scratch(&scratch);
-  if (e != cudaSuccess) return SMAT_ERR_CUDA;
-  cudaStream_t s = (cudaStream_t)stream;
-  unsigned char *sc = (unsigned char *)scratch;
-  switch (dtype) {
-    case SMAT_F64: e = merge_noalloc_typed<double>(m, nnz, rowptr, colidx, vals, alpha, x, beta, y, sc, s); break;
-    case SMAT_F32: e = merge_noalloc_typed<float>(m, nnz, rowptr, colidx, vals, alpha, x, beta, y, sc, s); break;
-    default: e = merge_noalloc_typed<__nv_bfloat16>(m, nnz, rowptr, colidx, vals, alpha, x, beta, y, sc, s); break;
-  }
-  return e == cudaSuccess ? SMAT_OK : SMAT_ERR_CUDA;
-}
