@@ -36,7 +36,7 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    return _sources() + [p for d, e in ((CSRC, "*.h"), (CSRC, "*.cuh"), (INCLUDE, "*.h")) for p in glob.glob(os.path.join(d, e))]
 
 
 def up_to_date() -> bool:

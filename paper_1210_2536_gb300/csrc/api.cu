@@ -384,6 +384,27 @@ void feature_vector(const smat_features_t &f, float out[12]) {
 // ---------------------------------------------------------------------------
 // Format construction (Sec. 2.1).
 // ---------------------------------------------------------------------------
+void free_row_ends(RowEnds &re) {
+  dev_free(re.ends); dev_free(re.ord); dev_free(re.row);
+  re = RowEnds{};
+}
+
+// Allocates and fills the row ends of a list of n entries in `rows` rows (see
+// launch_row_ends); with_row: the row of every row end is stored too.
+smat_status_t build_row_ends(const smat_s *h, RowEnds &re, int64_t n, int64_t rows, bool with_row,
+                             const int32_t *start32, const long long *start64, const long long *ordinal,
+                             cudaStream_t s) {
+  if (n <= 0) return SMAT_OK;
+  void *p = nullptr;
+  const size_t words = row_ends_words(n);
+  TRY(dev_alloc(&p, words * 4)); re.ends = (unsigned *)p;
+  TRY(dev_alloc(&p, words / 8 * 4)); re.ord = (int32_t *)p;
+  if (with_row) { TRY(dev_alloc(&p, (size_t)rows * 4)); re.row = (int32_t *)p; }
+  TRY(cudaMemsetAsync(re.ends, 0, words * 4, s));
+  TRY(launch_row_ends(re, h->m, start32, start64, ordinal, s));
+  return SMAT_OK;
+}
+
 void free_format(smat_s *h, int fmt) {
   if (fmt == SMAT_FMT_ELL) {
     dev_free(h->ell_col); dev_free(h->ell_val);
@@ -392,11 +413,13 @@ void free_format(smat_s *h, int fmt) {
     dev_free(h->dia_off); dev_free(h->dia_val);
     h->dia_off = nullptr; h->dia_val = nullptr; h->dia_nd = 0;
   } else if (fmt == SMAT_FMT_COO) {
-    dev_free(h->coo_row); dev_free(h->coo_empty);
-    h->coo_row = nullptr; h->coo_empty = nullptr; h->coo_nempty = 0;
+    free_row_ends(h->coo);
+    dev_free(h->coo_empty);
+    h->coo_empty = nullptr; h->coo_nempty = 0;
   } else if (fmt == SMAT_FMT_HYB) {
-    dev_free(h->hyb_ecol); dev_free(h->hyb_eval); dev_free(h->hyb_crow); dev_free(h->hyb_ccol); dev_free(h->hyb_cval);
-    h->hyb_ecol = h->hyb_crow = h->hyb_ccol = nullptr; h->hyb_eval = h->hyb_cval = nullptr; h->hyb_built = false;
+    dev_free(h->hyb_ecol); dev_free(h->hyb_eval); dev_free(h->hyb_ccol); dev_free(h->hyb_cval);
+    free_row_ends(h->hyb);
+    h->hyb_ecol = h->hyb_ccol = nullptr; h->hyb_eval = h->hyb_cval = nullptr; h->hyb_built = false;
   } else if (fmt == SMAT_FMT_SELL) {  // the layout (perm, width, slice pointers) stays
     dev_free(h->sell_col); dev_free(h->sell_val);
     h->sell_col = nullptr; h->sell_val = nullptr;
@@ -406,10 +429,11 @@ void free_format(smat_s *h, int fmt) {
     h->bcsr_cb = 0;
   } else if (fmt == SMAT_FMT_SPLIT) {
     for (int32_t **p : {&h->split_lchunk, &h->split_lrows, &h->split_crow, &h->split_cstart, &h->split_cend,
-                        &h->split_srow, &h->split_scol, &h->split_empty}) {
+                        &h->split_scol, &h->split_empty}) {
       dev_free(*p);
       *p = nullptr;
     }
+    free_row_ends(h->split);
     dev_free(h->split_sval); dev_free(h->split_part);
     h->split_sval = h->split_part = nullptr;
     h->split_built = false;
@@ -661,12 +685,23 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
     return measure_batch_width(h, SMAT_V_DIA, s);
   }
   if (fmt == SMAT_FMT_COO) {
-    if (h->coo_row || h->coo_empty) return SMAT_OK;
-    void *r = nullptr;
+    if (h->coo.ends || h->coo_empty) return SMAT_OK;
+    struct Undo {  // a failed build leaves no half-built format behind
+      smat_s *h; bool armed = true;
+      ~Undo() { if (armed) free_format(h, SMAT_FMT_COO); }
+    } undo{h};
     if (h->nnz > 0) {
-      TRY(dev_alloc(&r, (size_t)h->nnz * 4));
-      h->coo_row = (int32_t *)r;
-      TRY(launch_to_coo(h, h->coo_row, s));
+      // with empty rows the n-th row end is not row n's: number the others
+      const bool number = h->f.empty_rows > 0;
+      DevBuf flag(s), ord(s);
+      if (number) {
+        TRY(flag.alloc((size_t)h->m * 8));
+        TRY(ord.alloc((size_t)(h->m + 1) * 8));
+        TRY(launch_nonempty_rows(h, flag.as<long long>(), s));
+        TRY(exclusive_scan(flag.as<long long>(), h->m, ord.as<long long>(), s));
+      }
+      TRYS(build_row_ends(h, h->coo, h->nnz, h->m - h->f.empty_rows, number, h->rowptr, nullptr,
+                          number ? ord.as<long long>() : nullptr, s));
     }
     if (h->f.empty_rows > 0) {
       void *l = nullptr;
@@ -679,6 +714,7 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       TRY(launch_empty_rows(h, h->coo_empty, cnt.as<int>(), s));
       TRY(cudaStreamSynchronize(s));
     }
+    undo.armed = false;
     return SMAT_OK;
   }
   if (fmt == SMAT_FMT_HYB || fmt == SMAT_FMT_SELL || fmt == SMAT_FMT_BCSR || fmt == SMAT_FMT_SPLIT) {
@@ -697,7 +733,6 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       const int64_t K = h->hyb_K, nc = h->hyb_ncoo;
       TRY(dev_alloc(&p, (size_t)(K * h->P) * 4)); h->hyb_ecol = (int32_t *)p;
       TRY(dev_alloc(&p, (size_t)(K * h->P) * h->esz)); h->hyb_eval = p;
-      TRY(dev_alloc(&p, (size_t)nc * 4)); h->hyb_crow = (int32_t *)p;
       TRY(dev_alloc(&p, (size_t)nc * 4)); h->hyb_ccol = (int32_t *)p;
       TRY(dev_alloc(&p, (size_t)nc * h->esz)); h->hyb_cval = p;
       DevBuf cnt(s), off(s);
@@ -705,7 +740,16 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       TRY(off.alloc((size_t)(h->m + 1) * 8));
       TRY(launch_hyb_tail_counts(h, K, cnt.as<long long>(), s));
       TRY(exclusive_scan(cnt.as<long long>(), h->m, off.as<long long>(), s));
-      TRY(launch_to_hyb(h, K, off.as<long long>(), h->hyb_ecol, h->hyb_eval, h->hyb_crow, h->hyb_ccol, h->hyb_cval, s));
+      TRY(launch_to_hyb(h, K, off.as<long long>(), h->hyb_ecol, h->hyb_eval, h->hyb_ccol, h->hyb_cval, s));
+      if (nc > 0) {
+        DevBuf ord(s);
+        TRY(ord.alloc((size_t)(h->m + 1) * 8));
+        TRY(launch_nonzero(cnt.as<long long>(), h->m, cnt.as<long long>(), s));
+        TRY(exclusive_scan(cnt.as<long long>(), h->m, ord.as<long long>(), s));
+        int64_t tails = 0;
+        for (int64_t k = K + 1; k < (int64_t)h->hist.size(); ++k) tails += h->hist[(size_t)k];
+        TRYS(build_row_ends(h, h->hyb, nc, tails, true, nullptr, off.as<long long>(), ord.as<long long>(), s));
+      }
       TRY(cudaStreamSynchronize(s));
       h->hyb_built = true;
     } else if (fmt == SMAT_FMT_SELL) {
@@ -722,7 +766,6 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       TRY(dev_alloc(&p, nc * 4)); h->split_crow = (int32_t *)p;
       TRY(dev_alloc(&p, nc * 4)); h->split_cstart = (int32_t *)p;
       TRY(dev_alloc(&p, nc * 4)); h->split_cend = (int32_t *)p;
-      TRY(dev_alloc(&p, ns * 4)); h->split_srow = (int32_t *)p;
       TRY(dev_alloc(&p, ns * 4)); h->split_scol = (int32_t *)p;
       TRY(dev_alloc(&p, ns * h->esz)); h->split_sval = p;
       TRY(dev_alloc(&p, ne * 4)); h->split_empty = (int32_t *)p;
@@ -735,6 +778,9 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       TRY(launch_split_counts(h, c, c + M, c + 2 * M, c + 3 * M, s));
       for (int k = 0; k < 4; ++k) TRY(exclusive_scan(c + k * M, (long long)M, q + k * (M + 1), s));
       TRY(launch_split_fill(h, q, q + (M + 1), q + 2 * (M + 1), q + 3 * (M + 1), s));
+      TRY(launch_nonzero(c + 2 * M, h->m, c, s));
+      TRY(exclusive_scan(c, (long long)M, q, s));  // the long rows' numbers are no longer needed
+      TRYS(build_row_ends(h, h->split, h->split_ns, h->m - h->split_ne - h->split_nl, true, nullptr, q + 2 * (M + 1), q, s));
       TRY(cudaStreamSynchronize(s));
       h->split_built = true;
     } else {
@@ -825,7 +871,7 @@ bool variant_ready(const smat_s *h, int v) {
   if (v == SMAT_V_CSR_MERGE && h->m > 0 && !h->flat_row) return false;
   if (fmt == SMAT_FMT_ELL && !h->ell_val) return false;
   if (fmt == SMAT_FMT_DIA && !h->dia_val) return false;
-  if (fmt == SMAT_FMT_COO && !h->coo_row && !(h->nnz == 0)) return false;
+  if (fmt == SMAT_FMT_COO && !h->coo.ends && !(h->nnz == 0)) return false;
   if (fmt == SMAT_FMT_COO && h->f.empty_rows > 0 && !h->coo_empty) return false;
   if (fmt == SMAT_FMT_HYB && !h->hyb_built) return false;
   if (fmt == SMAT_FMT_SELL && !h->sell_val) return false;
@@ -1585,7 +1631,7 @@ smat_status_t smat_format_dims(smat_handle_t h, smat_format_t fmt, int64_t dims[
   switch (fmt) {
     case SMAT_FMT_ELL: if (!h->ell_val) return SMAT_ERR_UNSUPPORTED; dims[0] = h->ell_K; dims[1] = h->P; break;
     case SMAT_FMT_DIA: if (!h->dia_val) return SMAT_ERR_UNSUPPORTED; dims[0] = h->dia_nd; dims[1] = h->P; break;
-    case SMAT_FMT_COO: if (!h->coo_row && h->nnz > 0) return SMAT_ERR_UNSUPPORTED; dims[0] = h->nnz; dims[1] = 0; break;
+    case SMAT_FMT_COO: if (!h->coo.ends && h->nnz > 0) return SMAT_ERR_UNSUPPORTED; dims[0] = h->nnz; dims[1] = 0; break;
     case SMAT_FMT_CSR: dims[0] = h->m; dims[1] = h->nnz; break;
     case SMAT_FMT_HYB: if (!h->hyb_built) return SMAT_ERR_UNSUPPORTED; dims[0] = h->hyb_K; dims[1] = h->hyb_ncoo; break;
     case SMAT_FMT_SELL: if (!h->sell_val) return SMAT_ERR_UNSUPPORTED; dims[0] = h->sell_ns; dims[1] = h->sell_slots; break;
@@ -1594,6 +1640,16 @@ smat_status_t smat_format_dims(smat_handle_t h, smat_format_t fmt, int64_t dims[
     default: return SMAT_ERR_INVALID_ARG;
   }
   return SMAT_OK;
+}
+
+// The row index of each of a list's n entries, to host or device memory.
+static cudaError_t export_rows(const RowEnds &re, int64_t n, int32_t *out) {
+  if (n <= 0) return cudaSuccess;
+  DevBuf row(0);
+  cudaError_t e = row.alloc((size_t)n * 4);
+  if (e == cudaSuccess) e = launch_expand_rows(re, n, row.as<int32_t>(), 0);
+  if (e == cudaSuccess) e = cudaMemcpy(out, row.p, (size_t)n * 4, cudaMemcpyDefault);
+  return e;
 }
 
 smat_status_t smat_export_format(smat_handle_t h, smat_format_t fmt, int32_t *idx, void *val) {
@@ -1613,13 +1669,13 @@ smat_status_t smat_export_format(smat_handle_t h, smat_format_t fmt, int32_t *id
       break;
     case SMAT_FMT_COO:
       if (!idx) return SMAT_ERR_INVALID_ARG;
-      if (h->nnz > 0) TRY(cudaMemcpy(idx, h->coo_row, (size_t)h->nnz * 4, cudaMemcpyDefault));
+      TRY(export_rows(h->coo, h->nnz, idx));
       break;
     case SMAT_FMT_HYB: {
       if (!idx || !val) return SMAT_ERR_INVALID_ARG;
       const size_t ne = (size_t)(h->hyb_K * h->P), nc = (size_t)h->hyb_ncoo;
       if (ne) TRY(cudaMemcpy(idx, h->hyb_ecol, ne * 4, cudaMemcpyDefault));
-      if (nc) TRY(cudaMemcpy(idx + ne, h->hyb_crow, nc * 4, cudaMemcpyDefault));
+      TRY(export_rows(h->hyb, (int64_t)nc, idx + ne));
       if (nc) TRY(cudaMemcpy(idx + ne + nc, h->hyb_ccol, nc * 4, cudaMemcpyDefault));
       if (ne) TRY(cudaMemcpy(val, h->hyb_eval, ne * h->esz, cudaMemcpyDefault));
       if (nc) TRY(cudaMemcpy((char *)val + ne * h->esz, h->hyb_cval, nc * h->esz, cudaMemcpyDefault));
@@ -1645,7 +1701,7 @@ smat_status_t smat_export_format(smat_handle_t h, smat_format_t fmt, int32_t *id
       if (nc) TRY(cudaMemcpy(idx, h->split_crow, nc * 4, cudaMemcpyDefault));
       if (nc) TRY(cudaMemcpy(idx + nc, h->split_cstart, nc * 4, cudaMemcpyDefault));
       if (nc) TRY(cudaMemcpy(idx + 2 * nc, h->split_cend, nc * 4, cudaMemcpyDefault));
-      if (ns) TRY(cudaMemcpy(idx + 3 * nc, h->split_srow, ns * 4, cudaMemcpyDefault));
+      TRY(export_rows(h->split, (int64_t)ns, idx + 3 * nc));
       if (ns) TRY(cudaMemcpy(idx + 3 * nc + ns, h->split_scol, ns * 4, cudaMemcpyDefault));
       if (ns) TRY(cudaMemcpy(val, h->split_sval, ns * h->esz, cudaMemcpyDefault));
     } break;

@@ -23,33 +23,52 @@ template <> struct Bits<8> { typedef unsigned long long T; };
 template <> struct Bits<4> { typedef unsigned int T; };
 template <> struct Bits<2> { typedef unsigned short T; };
 
-__device__ __forceinline__ int row_lane_of(int start_of_my_row, long long k) {
-  int L = 0;
-#pragma unroll
-  for (int step = 16; step > 0; step >>= 1) {
-    int cand = L + step;
-    int sc = __shfl_sync(FULL, start_of_my_row, cand & 31);
-    if (cand < 32 && (long long)sc <= k) L = cand;
+// Row ends of a list: a thread per row marks its last entry, and writes its
+// ordinal for the tiles of 256 entries that start in it (a warp together where
+// they are many) and its row for the ordinal.
+template <typename S>
+__global__ void __launch_bounds__(256) row_ends_kernel(const S *__restrict__ start, const long long *__restrict__ ordinal,
+                                                       long long m, RowEnds re) {
+  const int lane = threadIdx.x & 31;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long r0 = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; r0 < m; r0 += stride) {
+    const long long r = r0 + lane;
+    long long t0 = 0, t1 = 0;  // the tiles that start in row r
+    int ord = 0;
+    if (r < m) {
+      const long long s = start[r], e = start[r + 1];
+      if (s < e) {
+        ord = ordinal ? (int)ordinal[r] : (int)r;
+        atomicOr(&re.ends[(e - 1) >> 5], 1u << ((e - 1) & 31));
+        if (re.row) re.row[ord] = (int32_t)r;
+        t0 = (s + 255) >> 8;
+        t1 = ((e - 1) >> 8) + 1;
+      }
+    }
+    const bool many = t1 - t0 > 8;
+    if (!many)
+      for (long long t = t0; t < t1; ++t) re.ord[t] = ord;
+    for (unsigned left = __ballot_sync(FULL, many); left; left &= left - 1) {
+      const int src = __ffs(left) - 1;
+      const long long a = __shfl_sync(FULL, t0, src), b = __shfl_sync(FULL, t1, src);
+      const int o = __shfl_sync(FULL, ord, src);
+      for (long long t = a + lane; t < b; t += 32) re.ord[t] = o;
+    }
   }
-  return L;
 }
 
-// COO row indices: a warp expands 32 rows over their contiguous nonzero range.
-__global__ void to_coo_kernel(const int32_t *__restrict__ rowptr, long long m, int32_t *__restrict__ row) {
+// The row of every entry, from the row ends: a warp per tile.
+__global__ void __launch_bounds__(256) expand_rows_kernel(RowEnds re, long long n, int32_t *__restrict__ row) {
   const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long r0 = warp * 32; r0 < m; r0 += nwarps * 32) {
-    long long r = r0 + lane;
-    int s = 0x7fffffff, e = 0;
-    if (r < m) { s = rowptr[r]; e = rowptr[r + 1]; }
-    int rows = (int)min(32LL, m - r0);
-    long long gs = __shfl_sync(FULL, s, 0), ge = __shfl_sync(FULL, e, rows - 1);
-    for (long long base = gs; base < ge; base += 32) {
-      long long k = base + lane;
-      int L = row_lane_of(s, k);
-      if (k < ge) row[k] = (int32_t)(r0 + L);
-    }
+  const long long tile = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (tile * 256 >= n) return;
+  int ord = re.ord[tile];
+  for (int w = 0; w < 8; ++w) {
+    const long long k = tile * 256 + w * 32 + lane;
+    const unsigned ends = re.ends[tile * 8 + w];
+    const int o = ord + __popc(ends & ((1u << lane) - 1u));
+    if (k < n) row[k] = re.row ? re.row[o] : o;
+    ord += __popc(ends);
   }
 }
 
@@ -57,6 +76,12 @@ __global__ void empty_rows_kernel(const int32_t *__restrict__ rowptr, long long 
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
        i += (long long)gridDim.x * blockDim.x)
     if (rowptr[i + 1] == rowptr[i]) list[atomicAdd(count, 1)] = (int32_t)i;
+}
+
+__global__ void nonempty_rows_kernel(const int32_t *__restrict__ rowptr, long long m, long long *__restrict__ flag) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
+       i += (long long)gridDim.x * blockDim.x)
+    flag[i] = rowptr[i + 1] > rowptr[i];
 }
 
 // ELL: thread per row (and per pad row up to P).
@@ -129,15 +154,32 @@ int grid_for(long long work, int block, int max_blocks) {
 
 }  // namespace
 
-cudaError_t launch_to_coo(const smat_s *h, int32_t *row, cudaStream_t s) {
-  if (h->m <= 0 || h->nnz <= 0) return cudaSuccess;
-  to_coo_kernel<<<grid_for((h->m + 31) / 32 * 32, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, row);
+size_t row_ends_words(int64_t n) { return (size_t)((n + 255) / 256 * 8); }
+
+cudaError_t launch_row_ends(const RowEnds &re, int64_t m, const int32_t *start32, const long long *start64,
+                            const long long *ordinal, cudaStream_t s) {
+  if (m <= 0) return cudaSuccess;
+  const int g = grid_for(m, 256, 152 * 16);
+  if (start32) row_ends_kernel<<<g, 256, 0, s>>>(start32, ordinal, m, re);
+  else row_ends_kernel<<<g, 256, 0, s>>>(start64, ordinal, m, re);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_expand_rows(const RowEnds &re, int64_t n, int32_t *row, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  expand_rows_kernel<<<(unsigned)((n + 2047) / 2048), 256, 0, s>>>(re, n, row);
   return cudaGetLastError();
 }
 
 cudaError_t launch_empty_rows(const smat_s *h, int32_t *list, int *d_count, cudaStream_t s) {
   if (h->m <= 0) return cudaSuccess;
   empty_rows_kernel<<<grid_for(h->m, 256, 152 * 8), 256, 0, s>>>(h->rowptr, h->m, list, d_count);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_nonempty_rows(const smat_s *h, long long *flag, cudaStream_t s) {
+  if (h->m <= 0) return cudaSuccess;
+  nonempty_rows_kernel<<<grid_for(h->m, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, flag);
   return cudaGetLastError();
 }
 

@@ -219,58 +219,6 @@ __global__ void __launch_bounds__(FLAT_NT) csr_flat_kernel(const int32_t *__rest
   }
 }
 
-// y[r] += alpha * (sum of the carries of row r): the carries of one row are
-// consecutive.  A warp takes 32 of them and adds up the runs that start among
-// them (a segmented scan); a run that reaches past them is followed by the
-// whole warp, 128 carries at a time, so that a row of millions of entries does
-// not wait for one thread.
-template <typename T, int MODE>
-__global__ void __launch_bounds__(256) flat_carry_kernel(const int32_t *__restrict__ carry_row,
-                                                         const T *__restrict__ carry_val, long long ntiles,
-                                                         Epi<T, MODE> ep, T *__restrict__ y) {
-  griddep_wait();
-  const int lane = threadIdx.x & 31;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; c0 < ntiles; c0 += stride) {
-    const long long c = c0 + lane;
-    const int row = c < ntiles ? carry_row[c] : -1;
-    T v = c < ntiles ? carry_val[c] : (T)0;
-    int prev = __shfl_up_sync(FULL, row, 1);
-    if (lane == 0) prev = c0 > 0 ? carry_row[c0 - 1] : -1;
-    const bool head = row >= 0 && row != prev;
-    // each head's sum over its run: the lanes after it with the same row
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const T up = __shfl_down_sync(FULL, v, o);
-      const int ur = __shfl_down_sync(FULL, row, o);
-      if (lane + o < 32 && ur == row) v = v + up;
-    }
-    // the run of the last head, when it goes on past these 32
-    const int last = __shfl_sync(FULL, row, 31);
-    const unsigned heads = __ballot_sync(FULL, head && row == last);
-    if (last >= 0 && heads) {
-      T more = 0;
-      for (long long q0 = c0 + 32; q0 < ntiles; q0 += 128) {
-        int rr[4];
-        T vv[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const long long q = q0 + 32 * k + lane;
-          rr[k] = q < ntiles ? carry_row[q] : -1;
-          vv[k] = q < ntiles ? carry_val[q] : (T)0;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) more = rr[k] == last ? more + vv[k] : more;
-        if (__shfl_sync(FULL, rr[3], 31) != last) break;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) more = more + __shfl_xor_sync(FULL, more, o);
-      if (lane == __ffs(heads) - 1) v = v + more;
-    }
-    if (head) y[row] = add_rn(y[row], MODE == EPI_COPY ? v : mul_rn(ep.alpha, v));
-  }
-}
-
 struct FlatArgs {
   const int32_t *rowptr, *col;
   const void *val;
@@ -303,7 +251,7 @@ cudaError_t flat_mode(const FlatArgs &a, typename Compute<V>::T alpha, const voi
                  (const V *)a.val, x, ep, y, a.nnz, (const int32_t *)a.tile_row, a.tiles, 1 << a.log2_chunks,
                  a.rows_pass ? 0 : 1, a.carry_row, (T *)a.carry_val);
   if (e != cudaSuccess || a.tiles == 1) return e;
-  return launch_pdl(flat_carry_kernel<T, MODE>, dim3(grid_for(a.tiles, 256, 152 * 8)), nt, 0, s,
+  return launch_pdl(carry_kernel<T, MODE>, dim3(grid_for(a.tiles, 256, 152 * 8)), nt, 0, s, (const int32_t *)nullptr,
                     (const int32_t *)a.carry_row, (const T *)a.carry_val, a.tiles, ep, y);
 }
 

@@ -137,7 +137,7 @@ template <typename B>
 __global__ void to_hyb_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
                               const B *__restrict__ val, long long m, long long P, long long K,
                               const long long *__restrict__ off, int32_t *__restrict__ ecol, B *__restrict__ eval,
-                              int32_t *__restrict__ crow, int32_t *__restrict__ ccol, B *__restrict__ cval) {
+                              int32_t *__restrict__ ccol, B *__restrict__ cval) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
     long long s = 0, rd = 0;
     if (i < m) { s = rowptr[i]; rd = rowptr[i + 1] - s; }
@@ -150,7 +150,6 @@ __global__ void to_hyb_kernel(const int32_t *__restrict__ rowptr, const int32_t 
     if (i < m)
       for (long long q = K; q < rd; ++q) {
         const long long o = off[i] + q - K;
-        crow[o] = (int32_t)i;
         ccol[o] = col[s + q];
         cval[o] = val[s + q];
       }
@@ -318,7 +317,7 @@ __global__ void split_fill_kernel(const int32_t *__restrict__ rowptr, const int3
                                   const long long *__restrict__ pc, const long long *__restrict__ ps,
                                   const long long *__restrict__ pe, int32_t *__restrict__ lrows,
                                   int32_t *__restrict__ lchunk, int32_t *__restrict__ crow, int32_t *__restrict__ cstart,
-                                  int32_t *__restrict__ cend, int32_t *__restrict__ srow, int32_t *__restrict__ scol,
+                                  int32_t *__restrict__ cend, int32_t *__restrict__ scol,
                                   B *__restrict__ sval, int32_t *__restrict__ empty) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
     const long long s0 = rowptr[i], e0 = rowptr[i + 1], rd = e0 - s0;
@@ -337,7 +336,6 @@ __global__ void split_fill_kernel(const int32_t *__restrict__ rowptr, const int3
     } else {
       long long o = ps[i];
       for (long long k = s0; k < e0; ++k, ++o) {
-        srow[o] = (int32_t)i;
         scol[o] = col[k];
         sval[o] = val[k];
       }
@@ -558,23 +556,34 @@ cudaError_t exclusive_scan(const long long *in, long long n, long long *out, cud
   return e;
 }
 
+__global__ void nonzero_kernel(const long long *__restrict__ count, long long m, long long *__restrict__ flag) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x)
+    flag[i] = count[i] > 0;
+}
+
+cudaError_t launch_nonzero(const long long *count, int64_t m, long long *flag, cudaStream_t s) {
+  if (m <= 0) return cudaSuccess;
+  nonzero_kernel<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(count, m, flag);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_hyb_tail_counts(const smat_s *h, int64_t K, long long *cnt, cudaStream_t s) {
   if (h->m <= 0) return cudaSuccess;
   hyb_tail_counts<<<grid_for(h->m, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, K, cnt);
   return cudaGetLastError();
 }
 
-cudaError_t launch_to_hyb(const smat_s *h, int64_t K, const long long *off, int32_t *ecol, void *eval, int32_t *crow,
+cudaError_t launch_to_hyb(const smat_s *h, int64_t K, const long long *off, int32_t *ecol, void *eval,
                           int32_t *ccol, void *cval, cudaStream_t s) {
   if (h->P <= 0) return cudaSuccess;
   const int g = grid_for(h->P, 256, 152 * 16);
   switch (h->esz) {
     case 8: to_hyb_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<8>::T *)h->val, h->m, h->P, K, off, ecol,
-                                              (Raw<8>::T *)eval, crow, ccol, (Raw<8>::T *)cval); break;
+                                              (Raw<8>::T *)eval, ccol, (Raw<8>::T *)cval); break;
     case 4: to_hyb_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<4>::T *)h->val, h->m, h->P, K, off, ecol,
-                                              (Raw<4>::T *)eval, crow, ccol, (Raw<4>::T *)cval); break;
+                                              (Raw<4>::T *)eval, ccol, (Raw<4>::T *)cval); break;
     default: to_hyb_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<2>::T *)h->val, h->m, h->P, K, off, ecol,
-                                               (Raw<2>::T *)eval, crow, ccol, (Raw<2>::T *)cval); break;
+                                               (Raw<2>::T *)eval, ccol, (Raw<2>::T *)cval); break;
   }
   return cudaGetLastError();
 }
@@ -665,15 +674,15 @@ cudaError_t launch_split_fill(const smat_s *h, const long long *pl, const long l
   switch (h->esz) {
     case 8: split_fill_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<8>::T *)h->val, h->m, pl, pc, ps, pe,
                                                   h->split_lrows, h->split_lchunk, h->split_crow, h->split_cstart,
-                                                  h->split_cend, h->split_srow, h->split_scol,
+                                                  h->split_cend, h->split_scol,
                                                   (Raw<8>::T *)h->split_sval, h->split_empty); break;
     case 4: split_fill_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<4>::T *)h->val, h->m, pl, pc, ps, pe,
                                                   h->split_lrows, h->split_lchunk, h->split_crow, h->split_cstart,
-                                                  h->split_cend, h->split_srow, h->split_scol,
+                                                  h->split_cend, h->split_scol,
                                                   (Raw<4>::T *)h->split_sval, h->split_empty); break;
     default: split_fill_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<2>::T *)h->val, h->m, pl, pc, ps, pe,
                                                    h->split_lrows, h->split_lchunk, h->split_crow, h->split_cstart,
-                                                   h->split_cend, h->split_srow, h->split_scol,
+                                                   h->split_cend, h->split_scol,
                                                    (Raw<2>::T *)h->split_sval, h->split_empty); break;
   }
   return cudaGetLastError();

@@ -53,6 +53,18 @@ Model &model();
 
 }  // namespace smat
 
+namespace smat {
+// Where the rows of a list of entries in row order end (COO, SPLIT's short
+// rows, HYB's tail): one bit per entry (ends: 32-bit words, bit k % 32 of word
+// k / 32; whole tiles of 256 entries, zero past the last), the number of row
+// ends before each tile (ord), and the row of every row end (row; nullptr when
+// the n-th row end is row n's).
+struct RowEnds {
+  unsigned *ends = nullptr;
+  int32_t *ord = nullptr, *row = nullptr;
+};
+}  // namespace smat
+
 // The handle.
 struct smat_s {
   int64_t m = 0, n = 0, nnz = 0;
@@ -90,14 +102,15 @@ struct smat_s {
   int64_t dia_nd = 0;
   int32_t *dia_off = nullptr;
   void *dia_val = nullptr;
-  // COO
-  int32_t *coo_row = nullptr;
+  // COO (columns and values are CSR's)
+  smat::RowEnds coo;
   int32_t *coo_empty = nullptr;  // list of empty rows (y = beta*y there)
   int64_t coo_nempty = 0;
 
   // HYB: ELL part (K x P) + COO part
   int64_t hyb_K = 0, hyb_ncoo = 0;
-  int32_t *hyb_ecol = nullptr, *hyb_crow = nullptr, *hyb_ccol = nullptr;
+  int32_t *hyb_ecol = nullptr, *hyb_ccol = nullptr;
+  smat::RowEnds hyb;
   void *hyb_eval = nullptr, *hyb_cval = nullptr;
   bool hyb_built = false;
   // SELL-32-sigma: layout (perm, width, slice pointers) then col / val
@@ -117,7 +130,8 @@ struct smat_s {
   int64_t split_nl = 0, split_nc = 0, split_ns = 0, split_ne = 0;
   int32_t *split_lchunk = nullptr;  // first chunk of each long row, nl + 1 values
   int32_t *split_lrows = nullptr, *split_crow = nullptr, *split_cstart = nullptr, *split_cend = nullptr;
-  int32_t *split_srow = nullptr, *split_scol = nullptr, *split_empty = nullptr;
+  int32_t *split_scol = nullptr, *split_empty = nullptr;
+  smat::RowEnds split;
   void *split_sval = nullptr, *split_part = nullptr;
   bool split_built = false;
   // measured layouts of HYB / SELL / BCSR / SPLIT (index v - SMAT_V_HYB):
@@ -178,8 +192,17 @@ cudaError_t launch_diag_reduce(const int *d_diag_cnt, int64_t m, int64_t n, int 
                                int tau_den, unsigned long long *d_counts, int32_t *d_offsets,
                                int64_t offsets_cap, cudaStream_t s);
 
-cudaError_t launch_to_coo(const smat_s *h, int32_t *row, cudaStream_t s);
+// Row ends (convert.cu).  List entries of row r: start[r] .. start[r + 1]
+// (32-bit rowptr or 64-bit scan), none for the rows without any; ordinal[r] =
+// rows with entries before r (nullptr: r).  launch_row_ends fills a zeroed
+// RowEnds; launch_expand_rows writes the row of each of the n entries.
+size_t row_ends_words(int64_t n);
+cudaError_t launch_row_ends(const RowEnds &re, int64_t m, const int32_t *start32, const long long *start64,
+                            const long long *ordinal, cudaStream_t s);
+cudaError_t launch_expand_rows(const RowEnds &re, int64_t n, int32_t *row, cudaStream_t s);
 cudaError_t launch_empty_rows(const smat_s *h, int32_t *list, int *d_count, cudaStream_t s);
+// flag[r] = 1 when row r has entries.
+cudaError_t launch_nonempty_rows(const smat_s *h, long long *flag, cudaStream_t s);
 cudaError_t launch_to_ell(const smat_s *h, int64_t K, int32_t *col, void *val, cudaStream_t s);
 cudaError_t launch_to_dia(const smat_s *h, const int32_t *d_off, int64_t nd, void *val,
                           cudaStream_t s);
@@ -189,7 +212,9 @@ cudaError_t launch_to_dia(const smat_s *h, const int32_t *d_off, int64_t nd, voi
 cudaError_t exclusive_scan(const long long *in, long long n, long long *out, cudaStream_t s);
 cudaError_t launch_hyb_tail_counts(const smat_s *h, int64_t K, long long *cnt, cudaStream_t s);
 cudaError_t launch_to_hyb(const smat_s *h, int64_t K, const long long *off, int32_t *ecol, void *eval,
-                          int32_t *crow, int32_t *ccol, void *cval, cudaStream_t s);
+                          int32_t *ccol, void *cval, cudaStream_t s);
+// flag[r] = 1 when count[r] > 0.
+cudaError_t launch_nonzero(const long long *count, int64_t m, long long *flag, cudaStream_t s);
 cudaError_t launch_sell_layout(const smat_s *h, int sigma, int32_t *perm, int32_t *width, long long *cnt,
                                cudaStream_t s);
 cudaError_t launch_to_sell(const smat_s *h, cudaStream_t s);

@@ -104,249 +104,110 @@ __global__ void __launch_bounds__(256) csr_vector_kernel(const int32_t *__restri
 }
 
 // ---------------------------------------------------------------------------
-// Tiled segmented reduction shared by merge-path CSR (K9) and COO (K12).
-// A CTA consumes a tile of NT*IPT items; each thread walks IPT consecutive
-// items, finishing the rows whose last nonzero it sees.  A thread's partial
-// sum of the row still open at its end flows into the first row finished by a
-// later thread.  Which thread that is follows from an integer max-scan of
-// "last thread that finished a row", so the floating-point work is one add
-// per partial (in thread order, hence deterministic) instead of a
-// floating-point scan -- FP64 adds are scarce on GB300.  The partial of the
-// row still open at the end of the tile becomes the tile's carry, added by a
-// fix-up kernel.
+// K12: COO (and SPLIT's short rows, HYB's tail): entries in row order, whose row
+// ends are marked by one bit each (RowEnds).  A warp takes a tile of 256
+// entries, 8 per lane: the columns and values (32-byte loads), the lane's 8
+// bits and the tile's first row number are loaded together and the gathers
+// follow at once.  A lane adds up its entries and closes a row at each mark;
+// the partial sums that cross lanes come from a segmented scan (shuffles); the
+// finished rows' sums go through shared memory, so that y is written with
+// contiguous lanes.  The row open at the tile's end becomes the tile's carry,
+// added by a second kernel.
+//
+// Bound by each SM's gathers in flight.  Before, a row index per entry was
+// loaded (4 of 16 or 12 bytes), every row end was a scattered store, and the
+// scan always took five FP64 steps.  us per product, before and now: power-law
+// 2e6 rows (28.7 M entries) FP64 153.6 -> 130.5, FP32 131.9 -> 111.4; 8e6 rows
+// BF16 520 -> 420; uniform 1e6 FP64 85.4 -> 75.7; 7-point 128^3 FP64 73 -> 50.
+// The bounds on CTAs per SM (48 and 40 registers) are the fastest of those
+// tried: 56 and 44 registers 136 and 115 us, six and eight CTAs spill.
 // ---------------------------------------------------------------------------
-// Fallback for tiles where a row spans many threads: a block-wide segmented
-// scan of (finished-a-row, partial) pairs in thread order (deterministic).
-template <typename T>
-struct SegPair {
-  int h;
-  T v;
-};
+constexpr int COO_NT = 256, COO_WARPS = COO_NT / 32;
+constexpr long long COO_TILE = 256;
+// Finished rows' sums staged per warp.  Staging a whole tile's (16 KB per CTA
+// in FP64) costs L1, whose lines hold the gathers in flight (power-law FP64 146
+// us against 131), and other kernels' room on the same SM.  In FP32 32 sums are
+// as fast as 64 alone (112 us) and better beside others: a batch of 16 FP32
+// matrices takes 66 us with 32, 71 with 64.
+template <typename T> constexpr int COO_SUMS = sizeof(T) == 8 ? 64 : 32;
 
-template <typename T>
-__device__ __forceinline__ SegPair<T> seg_combine(SegPair<T> a, SegPair<T> b) {
-  return SegPair<T>{a.h | b.h, b.h ? b.v : a.v + b.v};
-}
-
-template <typename T, int NT>
-__device__ __forceinline__ SegPair<T> block_seg_scan(SegPair<T> x, SegPair<T> *total) {
-  __shared__ int sh_h[NT / 32];
-  __shared__ T sh_v[NT / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  SegPair<T> inc = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int ph = __shfl_up_sync(FULL, inc.h, o);
-    const T pv = __shfl_up_sync(FULL, inc.v, o);
-    if (lane >= o) inc = seg_combine(SegPair<T>{ph, pv}, inc);
-  }
-  SegPair<T> exc{__shfl_up_sync(FULL, inc.h, 1), __shfl_up_sync(FULL, inc.v, 1)};
-  if (lane == 0) exc = SegPair<T>{0, (T)0};
-  if (lane == 31) { sh_h[w] = inc.h; sh_v[w] = inc.v; }
-  __syncthreads();
-  if (w == 0) {
-    SegPair<T> wi{lane < NT / 32 ? sh_h[lane] : 0, lane < NT / 32 ? sh_v[lane] : (T)0};
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int ph = __shfl_up_sync(FULL, wi.h, o);
-      const T pv = __shfl_up_sync(FULL, wi.v, o);
-      if (lane >= o) wi = seg_combine(SegPair<T>{ph, pv}, wi);
-    }
-    int eh = __shfl_up_sync(FULL, wi.h, 1);
-    T ev = __shfl_up_sync(FULL, wi.v, 1);
-    if (lane == 0) { eh = 0; ev = (T)0; }
-    if (lane < NT / 32) { sh_h[lane] = eh; sh_v[lane] = ev; }
-    if (lane == NT / 32 - 1) *total = wi;
-  }
-  __syncthreads();
-  return seg_combine(SegPair<T>{sh_h[w], sh_v[w]}, exc);
-}
-
-// h: this thread finished at least one row; c: its partial of the row open at
-// its end.  Returns the sum of the earlier partials that belong to this
-// thread's first finished row (meaningful when h); the last thread also
-// returns the tile's open partial in *open.  Runs of up to 16 partials are
-// summed serially (one add each); a tile with a longer run -- a row spanning
-// many threads -- uses the block-wide segmented scan instead.
-template <typename T, int NT>
-__device__ __forceinline__ T tile_carries(bool h, T c, T *open) {
-  __shared__ T s_c[NT];
-  __shared__ int s_wmax[NT / 32];
-  __shared__ SegPair<T> s_total;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  s_c[threadIdx.x] = c;
-  int v = h ? (int)threadIdx.x : -1;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int p = __shfl_up_sync(FULL, v, o);
-    if (lane >= o) v = max(v, p);
-  }
-  if (lane == 31) s_wmax[w] = v;
-  __syncthreads();
-  int before = -1;
-  for (int k = 0; k < w; ++k) before = max(before, s_wmax[k]);
-  const int incl = max(v, before);        // last thread <= me that finished a row
-  int excl = __shfl_up_sync(FULL, incl, 1);
-  if (lane == 0) excl = before;          // last thread < me that finished a row
-  const int run = h ? (int)threadIdx.x - max(excl, 0) : 0;
-  const int open_run = threadIdx.x == NT - 1 ? NT - max(incl, 0) : 0;
-  if (__syncthreads_or(run > 16 || open_run > 16)) {
-    const SegPair<T> in = block_seg_scan<T, NT>(SegPair<T>{h ? 1 : 0, c}, &s_total);
-    if (threadIdx.x == NT - 1) *open = s_total.v;
-    return in.v;
-  }
-  T in = 0;
-  if (h)
-    for (int j = max(excl, 0); j < (int)threadIdx.x; ++j) in += s_c[j];
-  if (threadIdx.x == NT - 1) {
-    T o = 0;
-    for (int j = max(incl, 0); j < NT; ++j) o += s_c[j];
-    *open = o;
-  }
-  return in;
-}
-
-// One chunk of up to IPT consecutive stored entries of a COO tile: each
-// product is one fused multiply-add into acc; where a row ends inside the
-// chunk (row[k+1] differs) its sum is written, except the thread's first row
-// end, which is held back in first_row / first_acc for the tile's carries.
-template <typename T, int IPT, int MODE>
-__device__ __forceinline__ void coo_chunk(const int (&r)[IPT], const int (&c)[IPT], const T (&v)[IPT], int r_next,
-                                          int valid, const T *__restrict__ x, const Epi<T, MODE> &ep, T *__restrict__ y,
-                                          T &acc, int &first_row, T &first_acc) {
-  T xv[IPT];
+template <typename V, typename T, int MODE>
+__device__ __forceinline__ void coo_tile(const RowEnds &re, const int32_t *__restrict__ col, const V *__restrict__ val,
+                                         const T *__restrict__ x, const Epi<T, MODE> &ep, T *__restrict__ y, long long n,
+                                         int32_t *carry_row, T *carry_val, long long tile, T *sum) {
+  constexpr int IPT = 8;
+  const int lane = threadIdx.x & 31;
+  const long long b0 = tile * COO_TILE;
+  if (b0 >= n) return;  // the whole warp
+  const int count = (int)min((long long)COO_TILE, n - b0);
+  const long long k0 = b0 + lane * IPT;
+  const int valid = max(0, min(IPT, count - lane * IPT));
+  const bool full = valid == IPT;
+  int c[IPT];
+  T v[IPT], xv[IPT];
+  load_i32_run<IPT>(col + k0, full, valid, c, 0);
+  const unsigned ends = __ldg(reinterpret_cast<const unsigned char *>(re.ends) + tile * 32 + lane);
+  const int o0 = __ldg(re.ord + tile);
+  load_val_run<V, IPT>(val + k0, full, valid, v);
 #pragma unroll
   for (int q = 0; q < IPT; ++q) xv[q] = q < valid ? __ldg(x + c[q]) : (T)0;
+  int before = __popc(ends);  // rows that end in earlier lanes
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int p = __shfl_up_sync(FULL, before, o);
+    if (lane >= o) before += p;
+  }
+  const int nrows = __shfl_sync(FULL, before, 31);
+  before -= __popc(ends);
+  const int row0 = lane < nrows && re.row ? __ldg(re.row + o0 + lane) : o0 + lane;
+  // xv[q] becomes the sum of the row that ends at entry q
+  T acc = 0;
 #pragma unroll
   for (int q = 0; q < IPT; ++q) {
-    if (q < valid) {
-      acc = fused(acc, v[q], xv[q]);
-      const int rn = q + 1 < IPT ? r[q + 1] : r_next;
-      if (rn != r[q]) {  // last stored entry of row r[q]
-        if (first_row < 0) {
-          first_row = r[q];
-          first_acc = acc;
-        } else {
-          y[r[q]] = ep(acc, y, (long long)r[q]);
-        }
-        acc = 0;
-      }
-    }
+    if (q < valid) acc = fused(acc, v[q], xv[q]);
+    xv[q] = acc;
+    if ((ends >> q) & 1u) acc = 0;
   }
-}
-
-// End of a COO tile [b0, tile_end): partial sums carried between the tile's
-// threads, the held-back first row ends, and the row left open at the tile's
-// end handed to the fix-up as (carry_row, carry_val)[tile].
-template <typename T, int NT, int MODE>
-__device__ __forceinline__ void coo_finish(long long tile_end, T acc, int first_row, T first_acc,
-                                           const Epi<T, MODE> &ep, T *__restrict__ y, long long nnz,
-                                           const int32_t *__restrict__ row, int32_t *carry_row, T *carry_val,
-                                           long long tile) {
-  T tile_open = 0;
-  const T incoming = tile_carries<T, NT>(first_row >= 0, acc, &tile_open);
-  if (first_row >= 0) y[first_row] = ep(incoming + first_acc, y, (long long)first_row);
-  if (threadIdx.x == NT - 1) {
-    // the row open at the end of the tile continues into the next tile
-    const long long kl = tile_end - 1;
-    const bool open = kl + 1 < nnz && __ldg(row + kl + 1) == __ldg(row + kl);
-    carry_row[tile] = open ? __ldg(row + kl) : -1;
-    carry_val[tile] = open ? tile_open : (T)0;
-  }
-}
-
-// K12: COO.  A CTA owns NT*CH*8 consecutive stored entries; thread t owns
-// CH*8 consecutive ones, read 8 at a time with 16-byte vector loads, and
-// accumulates them with one fused multiply-add each.  A row ends at entry k
-// when row[k+1] differs.  CH chunks per thread amortise the tile's fixed work
-// (carry resolution, barriers) over more entries.
-#ifndef SMAT_COO_MINB
-#define SMAT_COO_MINB 1
-#endif
-template <typename V, typename T, int NT, int CH, int MODE>
-__device__ __forceinline__ void coo_tile(const int32_t *__restrict__ row, const int32_t *__restrict__ col,
-                                         const V *__restrict__ val, const T *__restrict__ x, const Epi<T, MODE> &ep,
-                                         T *__restrict__ y, long long nnz, int32_t *carry_row, T *carry_val,
-                                         long long tile) {
-  constexpr int IPT = 8, TILE = NT * CH * IPT;
-  const long long b0 = tile * TILE;
-  const long long kt = b0 + (long long)threadIdx.x * (CH * IPT);
-  T acc = 0, first_acc = 0;
-  int first_row = -1;
-#ifdef SMAT_COO_UNROLL
+  T open;
+  const T in = warp_carries<T>(ends != 0, acc, &open);
+  for (int base = 0; base < nrows; base += COO_SUMS<T>) {  // the finished rows, COO_SUMS at a time
+    int at = before - base;
+    T *const first = sum + at;
+    const bool mine = ends && lane > 0 && (unsigned)at < (unsigned)COO_SUMS<T>;
 #pragma unroll
-#else
-#pragma unroll 1
-#endif
-  for (int ch = 0; ch < CH; ++ch) {
-    const long long k0 = kt + ch * IPT;
-    const int valid = k0 >= nnz ? 0 : (int)min((long long)IPT, nnz - k0);
-    if (CH == 1 && sizeof(V) == 8) {
-      // FP64: the row after this thread's entries is the next lane's first
-      // row (a lane past the end holds -1), so only lane 31 loads it: one L2
-      // sector request fewer per thread on a kernel bound by their rate
-      // (power-law SPLIT 176 -> 166.5 us).  The column and value loads go
-      // first so the gathers do not wait for the shuffle.  In FP32 the
-      // shuffle costs 8 registers (48 -> 56) and was 2-7 % slower.  Every
-      // lane reaches the shuffle before any leaves.
-      const bool full = valid == IPT;
-      int r[IPT], c[IPT];
-      T v[IPT];
-      load_i32_run<IPT>(col + k0, full, valid, c, 0);
-      load_val_run<V, IPT>(val + k0, full, valid, v);
-      load_i32_run<IPT>(row + k0, full, valid, r, -1);
-      int r_next = __shfl_down_sync(FULL, r[0], 1);
-      if ((threadIdx.x & 31) == 31) r_next = (k0 + IPT < nnz) ? __ldg(row + k0 + IPT) : -1;
-      if (valid == 0) break;
-      coo_chunk<T, IPT, MODE>(r, c, v, r_next, valid, x, ep, y, acc, first_row, first_acc);
-      continue;
+    for (int q = 0; q < IPT; ++q)
+      if ((ends >> q) & 1u) {
+        if ((unsigned)at < (unsigned)COO_SUMS<T>) sum[at] = xv[q];
+        ++at;
+      }
+    if (mine) *first = in + *first;
+    __syncwarp();
+    const int here = min(COO_SUMS<T>, nrows - base);
+    for (int i = lane; i < here; i += 32) {
+      const int row = base + i == lane ? row0 : re.row ? __ldg(re.row + o0 + base + i) : o0 + base + i;
+      y[row] = ep(sum[i], y, (long long)row);
     }
-    if (valid == 0) break;
-    const bool full = valid == IPT;
-    int r[IPT], c[IPT];
-    T v[IPT];
-    load_i32_run<IPT>(row + k0, full, valid, r, -1);
-    load_i32_run<IPT>(col + k0, full, valid, c, 0);
-    load_val_run<V, IPT>(val + k0, full, valid, v);
-    const int r_next = (k0 + IPT < nnz) ? __ldg(row + k0 + IPT) : -1;
-    coo_chunk<T, IPT, MODE>(r, c, v, r_next, valid, x, ep, y, acc, first_row, first_acc);
+    __syncwarp();
   }
-  coo_finish<T, NT, MODE>(min(b0 + TILE, nnz), acc, first_row, first_acc, ep, y, nnz, row, carry_row, carry_val,
-                          tile);
+  const unsigned last = __shfl_sync(FULL, ends, (count - 1) / IPT);
+  if (lane == 0) {
+    const bool opn = !((last >> ((count - 1) % IPT)) & 1u);
+    carry_row[tile] = opn ? o0 + nrows : -1;
+    carry_val[tile] = opn ? open : (T)0;
+  }
 }
 
-template <typename V, typename T, int NT, int CH, int MODE>
-__global__ void __launch_bounds__(NT, SMAT_COO_MINB) coo_kernel(const int32_t *__restrict__ row,
-                                                                const int32_t *__restrict__ col,
-                                                                const V *__restrict__ val, const T *__restrict__ x,
-                                                                Epi<T, MODE> ep, T *__restrict__ y, long long nnz,
-                                                                int32_t *carry_row, T *carry_val) {
+template <typename V, typename T, int MODE>
+__global__ void __launch_bounds__(COO_NT, sizeof(T) == 8 ? 5 : 6) coo_kernel(RowEnds re, const int32_t *__restrict__ col,
+                                                     const V *__restrict__ val, const T *__restrict__ x,
+                                                     Epi<T, MODE> ep, T *__restrict__ y, long long n,
+                                                     int32_t *carry_row, T *carry_val) {
   griddep_wait();
-  coo_tile<V, T, NT, CH, MODE>(row, col, val, x, ep, y, nnz, carry_row, carry_val, blockIdx.x);
+  __shared__ T s_sum[COO_WARPS][COO_SUMS<T>];
+  const int w = threadIdx.x >> 5;
+  coo_tile<V, T, MODE>(re, col, val, x, ep, y, n, carry_row, carry_val, (long long)blockIdx.x * COO_WARPS + w,
+                       s_sum[w]);
 }
-
-// COO launch shape (sweep knobs; these defaults measured fastest)
-#ifndef SMAT_COO_NT
-#define SMAT_COO_NT 256
-#endif
-#ifndef SMAT_COO_CH
-#define SMAT_COO_CH 1
-#endif
-constexpr int COO_NT = SMAT_COO_NT, COO_CH = SMAT_COO_CH, COO_IPT = 8 * SMAT_COO_CH;
-// SPLIT's short rows in tiles of one warp (32 threads x 8 entries) whose
-// carries are resolved with shuffles alone, or (0) in the COO kernel's
-// 256-thread tiles with a block-wide carry scan.
-#ifndef SMAT_SPLIT_WARP_TILES
-#define SMAT_SPLIT_WARP_TILES 1
-#endif
-constexpr bool SPLIT_WARP_TILES = SMAT_SPLIT_WARP_TILES != 0;
-constexpr long long SPLIT_TILE = SPLIT_WARP_TILES ? 32LL * 8 : (long long)COO_NT * COO_IPT;
-// The same choice for COO products (and HYB's COO tail).
-#ifndef SMAT_COO_WARP_TILES
-#define SMAT_COO_WARP_TILES 1
-#endif
-constexpr bool COO_WARP_TILES = SMAT_COO_WARP_TILES != 0;
-constexpr long long COO_TILE = COO_WARP_TILES ? 32LL * 8 : (long long)COO_NT * COO_IPT;
 
 // ---------------------------------------------------------------------------
 // SPLIT, long rows (at least SPLIT_L = 1024 entries; measured on power-law
@@ -404,74 +265,21 @@ __device__ __forceinline__ void split_chunk(long long c, const int32_t *__restri
 // blocks [nc, nc + tiles) are COO tiles of the short rows (the two sets
 // write disjoint rows).  One launch instead of two keeps the GPU full across
 // what was the boundary between them.
-// A COO tile of one warp: lane l owns the 8 stored entries at b0 + 8 l; rows
-// ending inside a lane's entries are written as in the block tiles, the
-// first one after the warp's carries, and the row open at the tile's end is
-// handed to the fix-up as (carry_row, carry_val)[tile].
 template <typename V, typename T, int MODE>
-__device__ __forceinline__ void coo_warp_tile(const int32_t *__restrict__ row, const int32_t *__restrict__ col,
-                                              const V *__restrict__ val, const T *__restrict__ x,
-                                              const Epi<T, MODE> &ep, T *__restrict__ y, long long nnz,
-                                              int32_t *carry_row, T *carry_val, long long tile) {
-  constexpr int IPT = 8;
-  const int lane = threadIdx.x & 31;
-  const long long b0 = tile * (32LL * IPT);
-  if (b0 >= nnz) return;  // the whole warp
-  const long long k0 = b0 + (long long)lane * IPT;
-  const int valid = k0 >= nnz ? 0 : (int)min((long long)IPT, nnz - k0);
-  const bool full = valid == IPT;
-  int r[IPT], c[IPT];
-  T v[IPT];
-  load_i32_run<IPT>(col + k0, full, valid, c, 0);
-  load_val_run<V, IPT>(val + k0, full, valid, v);
-  load_i32_run<IPT>(row + k0, full, valid, r, -1);
-  // the row after a lane's entries is the next lane's first row (a lane past
-  // the end holds -1); lane 31 loads it
-  int r_next = __shfl_down_sync(FULL, r[0], 1);
-  if (lane == 31) r_next = (k0 + IPT < nnz) ? __ldg(row + k0 + IPT) : -1;
-  T acc = 0, first_acc = 0;
-  int first_row = -1;
-  if (valid > 0) coo_chunk<T, IPT, MODE>(r, c, v, r_next, valid, x, ep, y, acc, first_row, first_acc);
-  T open;
-  const T incoming = warp_carries<T>(first_row >= 0, acc, &open);
-  if (first_row >= 0) y[first_row] = ep(incoming + first_acc, y, (long long)first_row);
-  if (lane == 31) {
-    const long long kl = min(b0 + 32LL * IPT, nnz) - 1;
-    const bool opn = kl + 1 < nnz && __ldg(row + kl + 1) == __ldg(row + kl);
-    carry_row[tile] = opn ? __ldg(row + kl) : -1;
-    carry_val[tile] = opn ? open : (T)0;
-  }
-}
-
-// COO products in warp tiles (coo_warp_tile), 8 tiles per 256-thread CTA.
-template <typename V, typename T, int MODE>
-__global__ void __launch_bounds__(COO_NT, SMAT_COO_MINB) coo_warp_kernel(const int32_t *__restrict__ row,
-                                                                     const int32_t *__restrict__ col,
-                                                                     const V *__restrict__ val,
-                                                                     const T *__restrict__ x, Epi<T, MODE> ep,
-                                                                     T *__restrict__ y, long long nnz,
-                                                                     int32_t *carry_row, T *carry_val) {
-  griddep_wait();
-  coo_warp_tile<V, T, MODE>(row, col, val, x, ep, y, nnz, carry_row, carry_val,
-                            (long long)blockIdx.x * (COO_NT / 32) + (threadIdx.x >> 5));
-}
-
-template <typename V, typename T, int MODE>
-__global__ void __launch_bounds__(COO_NT, SMAT_COO_MINB) split_main_kernel(
+__global__ void __launch_bounds__(COO_NT, sizeof(T) == 8 ? 5 : 6) split_main_kernel(
     const int32_t *__restrict__ cstart, const int32_t *__restrict__ cend, const int32_t *__restrict__ col,
-    const V *__restrict__ val, T *__restrict__ part, long long nc, const int32_t *__restrict__ srow,
-    const int32_t *__restrict__ scol, const V *__restrict__ sval, long long ns, const T *__restrict__ x,
-    Epi<T, MODE> ep, T *__restrict__ y, int32_t *carry_row, T *carry_val) {
+    const V *__restrict__ val, T *__restrict__ part, long long nc, RowEnds re, const int32_t *__restrict__ scol,
+    const V *__restrict__ sval, long long ns, const T *__restrict__ x, Epi<T, MODE> ep, T *__restrict__ y,
+    int32_t *carry_row, T *carry_val) {
   griddep_wait();
   static_assert(COO_NT == 256, "the chunk path assumes 256 threads");
+  __shared__ T s_sum[COO_WARPS][COO_SUMS<T>];
+  const int w = threadIdx.x >> 5;
   if ((long long)blockIdx.x < nc)
     split_chunk<V, T>(blockIdx.x, cstart, cend, col, val, x, part);
-  else if (SPLIT_WARP_TILES)
-    coo_warp_tile<V, T, MODE>(srow, scol, sval, x, ep, y, ns, carry_row, carry_val,
-                              ((long long)blockIdx.x - nc) * (COO_NT / 32) + (threadIdx.x >> 5));
   else
-    coo_tile<V, T, COO_NT, COO_CH, MODE>(srow, scol, sval, x, ep, y, ns, carry_row, carry_val,
-                                         (long long)blockIdx.x - nc);
+    coo_tile<V, T, MODE>(re, scol, sval, x, ep, y, ns, carry_row, carry_val,
+                         ((long long)blockIdx.x - nc) * COO_WARPS + w, s_sum[w]);
 }
 
 // A long row: its chunk sums added in chunk order, then the epilogue.
@@ -486,49 +294,24 @@ __device__ __forceinline__ void split_row(long long l, const int32_t *__restrict
   y[r] = ep(t, y, r);
 }
 
-// Fix-up: y[r] += alpha * (sum of the carries of row r), runs of equal rows
-// summed in tile order by the run's first entry.
-template <typename T, int MODE>
-__device__ __forceinline__ void carry_fixup(long long c, const int32_t *__restrict__ carry_row,
-                                            const T *__restrict__ carry_val, long long ntiles,
-                                            const Epi<T, MODE> &ep, T *__restrict__ y) {
-  const int r = carry_row[c];
-  if (r < 0 || (c > 0 && carry_row[c - 1] == r)) return;
-  T s = carry_val[c];
-  for (long long q = c + 1; q < ntiles && carry_row[q] == r; ++q) s = add_rn(s, carry_val[q]);
-  y[r] = add_rn(y[r], MODE == EPI_COPY ? s : mul_rn(ep.alpha, s));
-}
-
-template <typename T, int MODE>
-__global__ void carry_fixup_kernel(const int32_t *__restrict__ carry_row, const T *__restrict__ carry_val,
-                                   long long ntiles, Epi<T, MODE> ep, T *__restrict__ y) {
-  griddep_wait();
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < ntiles;
-       c += (long long)gridDim.x * blockDim.x)
-    carry_fixup<T, MODE>(c, carry_row, carry_val, ntiles, ep, y);
-}
-
 // SPLIT's closing pass over three disjoint sets of rows: the long rows
 // (chunk sums, epilogue), the carries of the short rows' COO tiles, and the
 // empty rows (y = beta y, or 0).
 template <typename T, int MODE>
 __global__ void split_finish_kernel(const int32_t *__restrict__ lrows, const int32_t *__restrict__ lchunk,
-                                    const T *__restrict__ part, long long nl, const int32_t *__restrict__ carry_row,
+                                    const T *__restrict__ part, long long nl, const int32_t *__restrict__ srows,
+                                    const int32_t *__restrict__ carry_row,
                                     const T *__restrict__ carry_val, long long ntiles,
                                     const int32_t *__restrict__ empty, long long ne, Epi<T, MODE> ep,
                                     T *__restrict__ y) {
   griddep_wait();
-  const long long total = nl + ntiles + ne;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    if (i < nl) {
-      split_row<T, MODE>(i, lrows, lchunk, part, ep, y);
-    } else if (i < nl + ntiles) {
-      carry_fixup<T, MODE>(i - nl, carry_row, carry_val, ntiles, ep, y);
-    } else {
-      const int r = empty[i - nl - ntiles];
-      y[r] = MODE == EPI_AXPBY ? mul_rn(ep.beta, y[r]) : (T)0;
-    }
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < nl; i += stride) split_row<T, MODE>(i, lrows, lchunk, part, ep, y);
+  for (long long c0 = first - (threadIdx.x & 31); c0 < ntiles; c0 += stride)
+    add_carries<T, MODE>(c0, srows, carry_row, carry_val, ntiles, ep, y);
+  for (long long i = first; i < ne; i += stride) {
+    const int r = empty[i];
+    y[r] = MODE == EPI_AXPBY ? mul_rn(ep.beta, y[r]) : (T)0;
   }
 }
 
@@ -600,22 +383,18 @@ int grid_for(long long work, int block, int max_blocks) {
   return (int)g;
 }
 
-// A COO product over (row, col, val) of length nnz, then the carry fix-up.
+// A COO product over nnz entries, then the carry fix-up.
 template <typename V, typename T, int MODE>
-cudaError_t launch_coo(const Scratch &sc, const int32_t *row, const int32_t *col, const V *val, const T *x,
+cudaError_t launch_coo(const Scratch &sc, const RowEnds &re, const int32_t *col, const V *val, const T *x,
                        const Epi<T, MODE> &ep, T *y, long long nnz, cudaStream_t s) {
   const long long tiles = (nnz + COO_TILE - 1) / COO_TILE;
   int32_t *crow = (int32_t *)sc.carry;
   T *cval = (T *)((char *)sc.carry + ((tiles * 4 + 15) / 16) * 16);
-  if (COO_WARP_TILES)
-    (void)launch_pdl(coo_warp_kernel<V, T, MODE>, dim3((unsigned)((tiles + COO_NT / 32 - 1) / (COO_NT / 32))), dim3(COO_NT), 0,
-        s, row, col, val, x, ep, y, nnz, crow, cval);
-  else
-    (void)launch_pdl(coo_kernel<V, T, COO_NT, COO_CH, MODE>, dim3((unsigned)tiles), dim3(COO_NT), 0, s, row, col, val, x, ep, y, nnz, crow, cval);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (tiles > 1) (void)launch_pdl(carry_fixup_kernel<T, MODE>, dim3(grid_for(tiles, 256, 152 * 8)), dim3(256), 0, s, crow, cval, tiles, ep, y);
-  return cudaGetLastError();
+  cudaError_t e = launch_pdl(coo_kernel<V, T, MODE>, dim3((unsigned)((tiles + COO_WARPS - 1) / COO_WARPS)), dim3(COO_NT),
+                             0, s, re, col, val, x, ep, y, nnz, crow, cval);
+  if (e != cudaSuccess || tiles <= 1) return e;
+  return launch_pdl(carry_kernel<T, MODE>, dim3(grid_for(tiles, 256, 152 * 8)), dim3(256), 0, s,
+                    (const int32_t *)re.row, (const int32_t *)crow, (const T *)cval, tiles, ep, y);
 }
 
 // ELL / DIA launches with a batch width U chosen at run time from 1..16/R.
@@ -718,7 +497,7 @@ cudaError_t spmv_mode(const smat_s *h, const Scratch &sc, int variant, typename 
         if (e != cudaSuccess) return e;
       }
       if (h->nnz == 0) break;
-      return launch_coo<V, T, MODE>(sc, h->coo_row, h->colidx, val, x, ep, y, h->nnz, s);
+      return launch_coo<V, T, MODE>(sc, h->coo, h->colidx, val, x, ep, y, h->nnz, s);
     }
     case SMAT_V_HYB: {
       // the ELL part writes every row (y = alpha*part + beta*y), then the COO
@@ -728,7 +507,7 @@ cudaError_t spmv_mode(const smat_s *h, const Scratch &sc, int variant, typename 
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess || h->hyb_ncoo == 0) return e;
       const Epi<T, EPI_AXPBY> add{alpha, (T)1};
-      return launch_coo<V, T, EPI_AXPBY>(sc, h->hyb_crow, h->hyb_ccol, (const V *)h->hyb_cval, x, add, y,
+      return launch_coo<V, T, EPI_AXPBY>(sc, h->hyb, h->hyb_ccol, (const V *)h->hyb_cval, x, add, y,
                                          h->hyb_ncoo, s);
     }
     case SMAT_V_SPLIT: {
@@ -736,21 +515,21 @@ cudaError_t spmv_mode(const smat_s *h, const Scratch &sc, int variant, typename 
       // short ones in one grid, then one pass for the long rows' sums, the
       // tiles' carries and the empty rows
       const long long nc = h->split_nc, ns = h->split_ns;
-      const long long tiles = (ns + SPLIT_TILE - 1) / SPLIT_TILE;
-      const long long tile_ctas = SPLIT_WARP_TILES ? (tiles + COO_NT / 32 - 1) / (COO_NT / 32) : tiles;
+      const long long tiles = (ns + COO_TILE - 1) / COO_TILE;
+      const long long tile_ctas = (tiles + COO_WARPS - 1) / COO_WARPS;
       int32_t *crow = (int32_t *)sc.carry;
       T *cval = (T *)((char *)sc.carry + ((tiles * 4 + 15) / 16) * 16);
       if (nc + tile_ctas > 0) {
         (void)launch_pdl(split_main_kernel<V, T, MODE>, dim3((unsigned)(nc + tile_ctas)), dim3(COO_NT), 0, s,
-            h->split_cstart, h->split_cend, h->colidx, val, (T *)sc.part, nc, h->split_srow, h->split_scol,
+            h->split_cstart, h->split_cend, h->colidx, val, (T *)sc.part, nc, h->split, h->split_scol,
             (const V *)h->split_sval, ns, x, ep, y, crow, cval);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
       }
       const long long nl = nc > 0 ? h->split_nl : 0, nt = tiles > 1 ? tiles : 0;
       if (nl + nt + h->split_ne > 0)
-        (void)launch_pdl(split_finish_kernel<T, MODE>, dim3(grid_for(nl + nt + h->split_ne, 256, 152 * 8)), dim3(256), 0, s,
-            h->split_lrows, h->split_lchunk, (const T *)sc.part, nl, crow, cval, nt, h->split_empty, h->split_ne, ep,
+        (void)launch_pdl(split_finish_kernel<T, MODE>, dim3(grid_for(std::max(nl, std::max(nt, (long long)h->split_ne)), 256, 152 * 8)), dim3(256), 0, s,
+            h->split_lrows, h->split_lchunk, (const T *)sc.part, nl, h->split.row, crow, cval, nt, h->split_empty, h->split_ne, ep,
             y);
     } break;
     default:
@@ -779,7 +558,7 @@ size_t carry_bytes_needed(const smat_s *h, int variant) {
   if (variant == SMAT_V_CSR_MERGE) tiles = flat_tiles(h->nnz);
   else if (variant == SMAT_V_COO) tiles = (h->nnz + COO_TILE - 1) / COO_TILE;
   else if (variant == SMAT_V_HYB) tiles = (h->hyb_ncoo + COO_TILE - 1) / COO_TILE;
-  else if (variant == SMAT_V_SPLIT) tiles = (h->split_ns + SPLIT_TILE - 1) / SPLIT_TILE;
+  else if (variant == SMAT_V_SPLIT) tiles = (h->split_ns + COO_TILE - 1) / COO_TILE;
   else return 0;
   size_t tsz = h->dtype == SMAT_F64 ? 8 : 4;
   return (size_t)((tiles * 4 + 15) / 16) * 16 + (size_t)tiles * tsz;
@@ -800,7 +579,7 @@ int spmv_launch_count(const smat_s *h, int variant) {
     return 1 + (h->hyb_ncoo > 0) + (tiles > 1);
   }
   if (variant == SMAT_V_SPLIT) {  // the main grid, then the closing pass when it has rows to do
-    const long long tiles = (h->split_ns + SPLIT_TILE - 1) / SPLIT_TILE;
+    const long long tiles = (h->split_ns + COO_TILE - 1) / COO_TILE;
     const long long nl = h->split_nc > 0 ? h->split_nl : 0, nt = tiles > 1 ? tiles : 0;
     return (h->split_nc + tiles > 0) + (nl + nt + h->split_ne > 0);
   }

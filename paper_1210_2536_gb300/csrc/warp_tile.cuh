@@ -86,23 +86,87 @@ __device__ __forceinline__ void load_val_run(const V *__restrict__ p, bool full,
 // end gets the sum at the lane before it: the partials of the row its first
 // row end closes.  *open is the sum at lane 31, the row left open at the
 // tile's end.  Shuffles only; fixed order.
+// Doubling steps that no lane needs any more (a row ended within reach of
+// every lane) are left out: in FP64 one step of a warp holds the SM's FP64 pipe
+// for 16 clocks, as long as one of the tile's eight multiply-adds.
 template <typename T>
 __device__ __forceinline__ T warp_carries(bool h, T c, T *open) {
   const int lane = threadIdx.x & 31;
-  int f = h ? 1 : 0;
+  unsigned reach = ~__ballot_sync(FULL, h);  // lanes that no row end in the last o lanes stops
   T v = c;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
+    if (reach == 0) break;
     const T vu = __shfl_up_sync(FULL, v, o);
-    const int fu = __shfl_up_sync(FULL, f, o);
-    if (lane >= o) {
-      if (!f) v = vu + v;
-      f |= fu;
-    }
+    if (lane >= o && ((reach >> lane) & 1u)) v = vu + v;
+    reach &= reach << o;
   }
   *open = __shfl_sync(FULL, v, 31);
   const T prev = __shfl_up_sync(FULL, v, 1);
   return lane == 0 ? (T)0 : prev;
+}
+
+// y[r] += alpha * (sum of the carries of row r), r = rows[carry_row] (rows
+// nullptr: carry_row itself); the carries of one row are consecutive.  A warp
+// takes the 32 carries at c0 and adds up the runs that start among them (a
+// segmented scan); a run that reaches past them is followed by the whole warp,
+// 128 carries at a time, so that a row of millions of entries does not wait for
+// one thread.
+template <typename T, int MODE>
+__device__ __forceinline__ void add_carries(long long c0, const int32_t *__restrict__ rows,
+                                            const int32_t *__restrict__ carry_row, const T *__restrict__ carry_val,
+                                            long long ntiles, const Epi<T, MODE> &ep, T *__restrict__ y) {
+  const int lane = threadIdx.x & 31;
+  const long long c = c0 + lane;
+  const int row = c < ntiles ? carry_row[c] : -1;
+  T v = c < ntiles ? carry_val[c] : (T)0;
+  int prev = __shfl_up_sync(FULL, row, 1);
+  if (lane == 0) prev = c0 > 0 ? carry_row[c0 - 1] : -1;
+  const bool head = row >= 0 && row != prev;
+  // each head's sum over its run: the lanes after it with the same row
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T up = __shfl_down_sync(FULL, v, o);
+    const int ur = __shfl_down_sync(FULL, row, o);
+    if (lane + o < 32 && ur == row) v = add_rn(v, up);
+  }
+  // the run of the last head, when it goes on past these 32
+  const int last = __shfl_sync(FULL, row, 31);
+  const unsigned heads = __ballot_sync(FULL, head && row == last);
+  if (last >= 0 && heads) {
+    T more = 0;
+    for (long long q0 = c0 + 32; q0 < ntiles; q0 += 128) {
+      int rr[4];
+      T vv[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const long long q = q0 + 32 * k + lane;
+        rr[k] = q < ntiles ? carry_row[q] : -1;
+        vv[k] = q < ntiles ? carry_val[q] : (T)0;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) more = rr[k] == last ? add_rn(more, vv[k]) : more;
+      if (__shfl_sync(FULL, rr[3], 31) != last) break;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) more = add_rn(more, __shfl_xor_sync(FULL, more, o));
+    if (lane == __ffs(heads) - 1) v = add_rn(v, more);
+  }
+  if (head) {
+    const long long r = rows ? rows[row] : row;
+    y[r] = add_rn(y[r], MODE == EPI_COPY ? v : mul_rn(ep.alpha, v));
+  }
+}
+
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256) carry_kernel(const int32_t *__restrict__ rows,
+                                                    const int32_t *__restrict__ carry_row,
+                                                    const T *__restrict__ carry_val, long long ntiles, Epi<T, MODE> ep,
+                                                    T *__restrict__ y) {
+  griddep_wait();
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long c0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); c0 < ntiles; c0 += stride)
+    add_carries<T, MODE>(c0, rows, carry_row, carry_val, ntiles, ep, y);
 }
 
 }  // namespace
