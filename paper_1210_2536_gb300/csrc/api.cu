@@ -298,56 +298,63 @@ smat_status_t compute_features(smat_s *h, cudaStream_t s) {
   f.m = h->m;
   f.n = h->n;
   f.nnz = h->nnz;
-  RowStats st{0ull, 0, h->m > 0 ? INT_MAX : 0, 0, 0};
-  if (h->m > 0) {
-    DevBuf d_st(s);
-    TRY(d_st.alloc(sizeof(RowStats)));
-    TRY(cudaMemcpyAsync(d_st.p, &st, sizeof(st), cudaMemcpyHostToDevice, s));
-    TRY(launch_row_stats(h->rowptr, h->m, d_st.as<RowStats>(), s));
-    TRY(cudaMemcpyAsync(&st, d_st.p, sizeof(st), cudaMemcpyDeviceToHost, s));
-    TRY(cudaStreamSynchronize(s));
-  }
-  f.max_rd = st.max_rd;
-  f.min_rd = st.min_rd;
-  f.empty_rows = st.empty_rows;
-  f.s2 = st.s2;
-  const int64_t hist_len = f.max_rd + 1;
-  h->hist.assign((size_t)hist_len, 0);
+  h->hist.assign(1, 0);
   h->dia_offsets.clear();
   h->dia_offsets_complete = false;
-  const int64_t nd_all = h->m + h->n - 1;
-  if (h->m > 0 && h->n > 0) {
-    DevBuf d_hist(s), d_cnt(s), d_counts(s), d_off(s);
-    TRY(d_hist.alloc((size_t)hist_len * sizeof(int)));
-    TRY(d_cnt.alloc((size_t)nd_all * sizeof(int)));
-    TRY(cudaMemsetAsync(d_hist.p, 0, (size_t)hist_len * sizeof(int), s));
-    TRY(cudaMemsetAsync(d_cnt.p, 0, (size_t)nd_all * sizeof(int), s));
-    TRY(launch_hist_diag(h->rowptr, h->colidx, h->m, d_hist.as<int>(), hist_len, d_cnt.as<int>(), s));
+  if (h->m > 0) {
+    // one block: the head and the offsets (read back together), the diagonals'
+    // counts, and the degrees of the long rows; three launches, one wait
+    const int64_t nd_all = h->n > 0 ? h->m + h->n - 1 : 0;
     // offsets are kept while DIA can still be admissible (Ndiags <= 20 aver_RD)
     int64_t cap = (int64_t)((__int128)h->fill_ratio_max * h->nnz / h->m) + 1;
-    cap = std::max<int64_t>(cap, 64);
-    cap = std::min<int64_t>(cap, nd_all);
-    TRY(d_counts.alloc(3 * sizeof(unsigned long long)));
-    TRY(d_off.alloc((size_t)cap * sizeof(int32_t)));
-    TRY(cudaMemsetAsync(d_counts.p, 0, 3 * sizeof(unsigned long long), s));
-    TRY(launch_diag_reduce(d_cnt.as<int>(), h->m, h->n, h->tau_num, h->tau_den,
-                           d_counts.as<unsigned long long>(), d_off.as<int32_t>(), cap, s));
-    unsigned long long counts[3];
-    std::vector<int> hist32((size_t)hist_len);
-    TRY(cudaMemcpyAsync(counts, d_counts.p, sizeof(counts), cudaMemcpyDeviceToHost, s));
-    TRY(cudaMemcpyAsync(hist32.data(), d_hist.p, (size_t)hist_len * sizeof(int), cudaMemcpyDeviceToHost, s));
+    cap = std::min<int64_t>(std::max<int64_t>(cap, 64), nd_all);
+    const int64_t read = std::min<int64_t>(cap, 4096);  // offsets read with the head
+    const auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t off_cap = sizeof(FeatureHead), off_cnt = up(off_cap + (size_t)cap * 4),
+                 off_long = off_cnt + up((size_t)nd_all * 4), total = off_long + (size_t)(h->nnz / HIST_LEN + 1) * 4;
+    DevBuf buf(s);
+    TRY(buf.alloc(total));
+    char *base = buf.as<char>();
+    FeatureHead *d_head = (FeatureHead *)base;
+    int32_t *d_off = (int32_t *)(base + off_cap), *d_long = (int32_t *)(base + off_long);
+    int *d_cnt = (int *)(base + off_cnt);
+    TRY(cudaMemsetAsync(base, 0, off_long, s));
+    TRY(launch_row_stats(h->rowptr, h->m, d_head, d_long, s));
+    if (nd_all > 0) {
+      TRY(launch_diag_count(h->rowptr, h->colidx, h->m, h->nnz, d_cnt, s));
+      TRY(launch_diag_reduce(d_cnt, h->m, h->n, h->tau_num, h->tau_den, d_head->counts, d_off, cap, s));
+    }
+    std::vector<char> host(off_cap + (size_t)read * 4);
+    TRY(cudaMemcpyAsync(host.data(), base, host.size(), cudaMemcpyDeviceToHost, s));
     TRY(cudaStreamSynchronize(s));
-    for (int64_t k = 0; k < hist_len; ++k) h->hist[(size_t)k] = hist32[(size_t)k];
-    f.ndiags = (int64_t)counts[0];
-    f.ntdiags = (int64_t)counts[1];
-    if ((int64_t)counts[2] <= cap) {
-      h->dia_offsets.resize((size_t)counts[2]);
-      TRY(cudaMemcpy(h->dia_offsets.data(), d_off.p, (size_t)counts[2] * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    FeatureHead head;
+    std::memcpy(&head, host.data(), sizeof(head));
+    f.max_rd = head.max_rd;
+    f.min_rd = INT_MAX - head.below_max;
+    f.empty_rows = head.empty_rows;
+    f.s2 = head.s2;
+    h->hist.assign((size_t)f.max_rd + 1, 0);
+    for (int64_t k = 0; k < HIST_LEN && k <= f.max_rd; ++k) h->hist[(size_t)k] = head.hist[k];
+    if (head.nlong > 0) {
+      std::vector<int32_t> lengths((size_t)head.nlong);
+      TRY(cudaMemcpyAsync(lengths.data(), d_long, lengths.size() * 4, cudaMemcpyDeviceToHost, s));
+      TRY(cudaStreamSynchronize(s));
+      for (int32_t rd : lengths) ++h->hist[(size_t)rd];
+    }
+    f.ndiags = (int64_t)head.counts[0];
+    f.ntdiags = (int64_t)head.counts[1];
+    const int64_t found = f.ndiags;
+    if (nd_all > 0 && found <= cap) {
+      h->dia_offsets.resize((size_t)found);
+      std::memcpy(h->dia_offsets.data(), host.data() + off_cap, (size_t)std::min(found, read) * 4);
+      if (found > read) {
+        TRY(cudaMemcpyAsync(h->dia_offsets.data() + read, d_off + read, (size_t)(found - read) * 4,
+                            cudaMemcpyDeviceToHost, s));
+        TRY(cudaStreamSynchronize(s));
+      }
       std::sort(h->dia_offsets.begin(), h->dia_offsets.end());
       h->dia_offsets_complete = true;
     }
-  } else if (h->m > 0) {
-    h->hist[0] = h->m;  // no columns: every row is empty
   }
   if (h->m > 0) {
     const double M = (double)h->m;

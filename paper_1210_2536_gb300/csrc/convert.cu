@@ -93,15 +93,13 @@ __global__ void to_ell_kernel(const int32_t *__restrict__ rowptr, const int32_t 
        i += (long long)gridDim.x * blockDim.x) {
     long long s = 0, rd = 0;
     if (i < m) { s = rowptr[i]; rd = rowptr[i + 1] - s; }
+#pragma unroll 8
     for (long long q = 0; q < K; ++q) {
-      long long pos = q * P + i;
-      if (q < rd) {
-        ecol[pos] = col[s + q];
-        eval[pos] = val[s + q];
-      } else {
-        ecol[pos] = -1;
-        eval[pos] = (B)0;
-      }
+      const long long pos = q * P + i;
+      const int c = q < rd ? col[s + q] : -1;
+      const B v = q < rd ? val[s + q] : (B)0;
+      ecol[pos] = c;
+      eval[pos] = v;
     }
   }
 }

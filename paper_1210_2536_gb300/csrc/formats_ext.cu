@@ -160,19 +160,31 @@ __global__ void to_hyb_kernel(const int32_t *__restrict__ rowptr, const int32_t 
 // SELL-C-sigma
 // ---------------------------------------------------------------------------
 // One block per window: each row's sorted position is the number of rows in
-// its window that are longer, or as long and earlier.
+// its window that are longer, or as long and earlier: the earlier ones at least
+// as long and the later ones longer, four lengths per shared load (only the
+// warp's own 32 rows need both tests).  As many threads as rows: 1024 for 256
+// rows, each comparing twice, took 61 us on 1e6 rows; 33 us now.
 __global__ void sell_sort_kernel(const int32_t *__restrict__ rowptr, long long m, int sigma, int32_t *__restrict__ perm) {
-  extern __shared__ int s_len[];
+  extern __shared__ __align__(16) int s_len[];  // sigma lengths, -1 past the last row
   const long long w0 = (long long)blockIdx.x * sigma;
   const int cnt = (int)(m - w0 < sigma ? m - w0 : sigma);
-  for (int q = threadIdx.x; q < cnt; q += blockDim.x) s_len[q] = rowptr[w0 + q + 1] - rowptr[w0 + q];
+  for (int q = threadIdx.x; q < sigma; q += blockDim.x) s_len[q] = q < cnt ? rowptr[w0 + q + 1] - rowptr[w0 + q] : -1;
   __syncthreads();
+  const int4 *len4 = reinterpret_cast<const int4 *>(s_len);
+  const int top = (cnt + 31) / 32 * 32;
   for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
-    const int lq = s_len[q];
+    const int lq = s_len[q], own = q & ~31;
     int rank = 0;
-    for (int t = 0; t < cnt; ++t) {
-      const int lt = s_len[t];
-      rank += (lt > lq) || (lt == lq && t < q);
+#pragma unroll 4
+    for (int t = 0; t < own / 4; ++t) {
+      const int4 l = len4[t];
+      rank += (l.x >= lq) + (l.y >= lq) + (l.z >= lq) + (l.w >= lq);
+    }
+    for (int t = own; t < own + 32; ++t) rank += (s_len[t] > lq) || (s_len[t] == lq && t < q);
+#pragma unroll 4
+    for (int t = own / 4 + 8; t < top / 4; ++t) {
+      const int4 l = len4[t];
+      rank += (l.x > lq) + (l.y > lq) + (l.z > lq) + (l.w > lq);
     }
     perm[w0 + rank] = (int32_t)(w0 + q);
   }
@@ -212,6 +224,7 @@ __global__ void to_sell_kernel(const int32_t *__restrict__ rowptr, const int32_t
     if (r >= 0) { k0 = rowptr[r]; len = rowptr[r + 1] - k0; }
     const long long base = sptr[sl] + (p % SELL_C);
     const int w = width[sl];
+#pragma unroll 8
     for (int j = 0; j < w; ++j) {
       const long long slot = base + (long long)j * SELL_C;
       const bool on = j < len;
@@ -545,14 +558,14 @@ cudaError_t exclusive_scan(const long long *in, long long n, long long *out, cud
   if (n <= 0) return cudaMemsetAsync(out, 0, sizeof(long long), s);
   const long long tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   void *sums = nullptr;
-  cudaError_t e = dev_alloc(&sums, (size_t)tiles * sizeof(long long));
+  cudaError_t e = tmp_alloc(&sums, (size_t)tiles * sizeof(long long), s);
   if (e != cudaSuccess) return e;
   scan_tile_sums<<<(unsigned)tiles, SCAN_NT, 0, s>>>(in, n, (long long *)sums);
   scan_tile_offsets<<<1, SCAN_NT, 0, s>>>((long long *)sums, tiles);
   scan_tiles<<<(unsigned)tiles, SCAN_NT, 0, s>>>(in, n, (const long long *)sums, out);
   e = cudaGetLastError();
+  tmp_free(sums, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  dev_free(sums);
   return e;
 }
 
@@ -592,7 +605,7 @@ cudaError_t launch_sell_layout(const smat_s *h, int sigma, int32_t *perm, int32_
                                cudaStream_t s) {
   if (h->m <= 0) return cudaSuccess;
   const long long windows = (h->m + sigma - 1) / sigma;
-  sell_sort_kernel<<<(unsigned)windows, 1024, (size_t)sigma * sizeof(int), s>>>(h->rowptr, h->m, sigma, perm);
+  sell_sort_kernel<<<(unsigned)windows, std::min(sigma, 1024), (size_t)sigma * sizeof(int), s>>>(h->rowptr, h->m, sigma, perm);
   const long long mp = (h->m + SELL_C - 1) / SELL_C * SELL_C;
   sell_width_kernel<<<grid_for(mp, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, mp, perm, width, cnt);
   return cudaGetLastError();

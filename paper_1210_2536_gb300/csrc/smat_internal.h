@@ -20,6 +20,9 @@ inline int64_t pitch_of(int64_t m) { return (m + 31) / 32 * 32; }
 // that makes a chosen allocation fail, for error-path tests.
 cudaError_t dev_alloc(void **p, size_t bytes);
 void dev_free(void *p);
+// Temporaries used on one stream only, allocated and freed in its order.
+cudaError_t tmp_alloc(void **p, size_t bytes, cudaStream_t s);
+void tmp_free(void *p, cudaStream_t s);
 
 // Plan cache (plan_cache.cu): the structural key, computed once per handle,
 // and the process-wide table of plans.
@@ -34,13 +37,17 @@ enum : int {
   ERRF_COL_ORDER = 4,  // columns not strictly increasing in a row
 };
 
-// Integer statistics of the row degrees (one pass over rowptr).
-struct RowStats {
-  unsigned long long s2;  // sum of rd^2
+// What feature extraction leaves on the device, all zero before it: integer
+// statistics and histogram of the row degrees, and the diagonals' counts.
+constexpr int HIST_LEN = 1024;
+struct FeatureHead {
+  unsigned long long s2;         // sum of rd^2
+  unsigned long long counts[2];  // occupied diagonals, "true" ones
   int max_rd;
-  int min_rd;
+  int below_max;  // INT_MAX - the smallest degree
   int empty_rows;
-  int pad;
+  int nlong;           // rows of HIST_LEN entries and more
+  int hist[HIST_LEN];  // rows of every shorter length
 };
 
 // Selector model (process-wide).
@@ -185,9 +192,9 @@ namespace smat {
 // words of one bit per stored entry (validate_starts_words of them).
 size_t validate_starts_words(int64_t nnz);
 cudaError_t launch_validate(const smat_s *h, int *d_flag, unsigned *d_starts, cudaStream_t s);
-cudaError_t launch_row_stats(const int32_t *rowptr, int64_t m, RowStats *d_stats, cudaStream_t s);
-cudaError_t launch_hist_diag(const int32_t *rowptr, const int32_t *colidx, int64_t m,
-                             int *d_hist, int64_t hist_len, int *d_diag_cnt, cudaStream_t s);
+cudaError_t launch_row_stats(const int32_t *rowptr, int64_t m, FeatureHead *head, int32_t *long_rows, cudaStream_t s);
+cudaError_t launch_diag_count(const int32_t *rowptr, const int32_t *colidx, int64_t m, int64_t nnz, int *d_diag_cnt,
+                              cudaStream_t s);
 cudaError_t launch_diag_reduce(const int *d_diag_cnt, int64_t m, int64_t n, int tau_num,
                                int tau_den, unsigned long long *d_counts, int32_t *d_offsets,
                                int64_t offsets_cap, cudaStream_t s);
