@@ -399,8 +399,7 @@ void free_row_ends(RowEnds &re) {
 // Allocates and fills the row ends of a list of n entries in `rows` rows (see
 // launch_row_ends); with_row: the row of every row end is stored too.
 smat_status_t build_row_ends(const smat_s *h, RowEnds &re, int64_t n, int64_t rows, bool with_row,
-                             const int32_t *start32, const long long *start64, const long long *ordinal,
-                             cudaStream_t s) {
+                             const int32_t *rowptr, const long long *scan, cudaStream_t s) {
   if (n <= 0) return SMAT_OK;
   void *p = nullptr;
   const size_t words = row_ends_words(n);
@@ -408,7 +407,7 @@ smat_status_t build_row_ends(const smat_s *h, RowEnds &re, int64_t n, int64_t ro
   TRY(dev_alloc(&p, words / 8 * 4)); re.ord = (int32_t *)p;
   if (with_row) { TRY(dev_alloc(&p, (size_t)rows * 4)); re.row = (int32_t *)p; }
   TRY(cudaMemsetAsync(re.ends, 0, words * 4, s));
-  TRY(launch_row_ends(re, h->m, start32, start64, ordinal, s));
+  TRY(launch_row_ends(re, h->m, rowptr, scan, s));
   return SMAT_OK;
 }
 
@@ -707,7 +706,7 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
         TRY(launch_nonempty_rows(h, flag.as<long long>(), s));
         TRY(exclusive_scan(flag.as<long long>(), h->m, ord.as<long long>(), s));
       }
-      TRYS(build_row_ends(h, h->coo, h->nnz, h->m - h->f.empty_rows, number, h->rowptr, nullptr,
+      TRYS(build_row_ends(h, h->coo, h->nnz, h->m - h->f.empty_rows, number, h->rowptr,
                           number ? ord.as<long long>() : nullptr, s));
     }
     if (h->f.empty_rows > 0) {
@@ -747,15 +746,12 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       TRY(off.alloc((size_t)(h->m + 1) * 8));
       TRY(launch_hyb_tail_counts(h, K, cnt.as<long long>(), s));
       TRY(exclusive_scan(cnt.as<long long>(), h->m, off.as<long long>(), s));
-      TRY(launch_to_hyb(h, K, off.as<long long>(), h->hyb_ecol, h->hyb_eval, h->hyb_ccol, h->hyb_cval, s));
+      TRY(launch_to_ell(h, K, h->hyb_ecol, h->hyb_eval, s));
       if (nc > 0) {
-        DevBuf ord(s);
-        TRY(ord.alloc((size_t)(h->m + 1) * 8));
-        TRY(launch_nonzero(cnt.as<long long>(), h->m, cnt.as<long long>(), s));
-        TRY(exclusive_scan(cnt.as<long long>(), h->m, ord.as<long long>(), s));
         int64_t tails = 0;
         for (int64_t k = K + 1; k < (int64_t)h->hist.size(); ++k) tails += h->hist[(size_t)k];
-        TRYS(build_row_ends(h, h->hyb, nc, tails, true, nullptr, off.as<long long>(), ord.as<long long>(), s));
+        TRYS(build_row_ends(h, h->hyb, nc, tails, true, nullptr, off.as<long long>(), s));
+        TRY(launch_list_copy(h, h->hyb, nc, off.as<long long>(), K, h->hyb_ccol, h->hyb_cval, s));
       }
       TRY(cudaStreamSynchronize(s));
       h->hyb_built = true;
@@ -779,15 +775,14 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
       TRY(dev_alloc(&p, nc * tsize(h))); h->split_part = p;
       DevBuf cnt(s), pre(s);
       const size_t M = (size_t)h->m;
-      TRY(cnt.alloc(4 * M * 8));
-      TRY(pre.alloc(4 * (M + 1) * 8));
-      long long *c = cnt.as<long long>(), *q = pre.as<long long>();
-      TRY(launch_split_counts(h, c, c + M, c + 2 * M, c + 3 * M, s));
-      for (int k = 0; k < 4; ++k) TRY(exclusive_scan(c + k * M, (long long)M, q + k * (M + 1), s));
-      TRY(launch_split_fill(h, q, q + (M + 1), q + 2 * (M + 1), q + 3 * (M + 1), s));
-      TRY(launch_nonzero(c + 2 * M, h->m, c, s));
-      TRY(exclusive_scan(c, (long long)M, q, s));  // the long rows' numbers are no longer needed
-      TRYS(build_row_ends(h, h->split, h->split_ns, h->m - h->split_ne - h->split_nl, true, nullptr, q + 2 * (M + 1), q, s));
+      TRY(cnt.alloc(3 * M * 8));
+      TRY(pre.alloc(3 * (M + 1) * 8));
+      long long *c = cnt.as<long long>(), *q = pre.as<long long>(), *q_short = q + (M + 1), *q_empty = q + 2 * (M + 1);
+      TRY(launch_split_counts(h, c, c + M, c + 2 * M, s));
+      for (int k = 0; k < 3; ++k) TRY(exclusive_scan(c + k * M, (long long)M, q + k * (M + 1), s));
+      TRY(launch_split_fill(h, q, q_empty, s));
+      TRYS(build_row_ends(h, h->split, h->split_ns, h->m - h->split_ne - h->split_nl, true, nullptr, q_short, s));
+      TRY(launch_list_copy(h, h->split, h->split_ns, q_short, 0, h->split_scol, h->split_sval, s));
       TRY(cudaStreamSynchronize(s));
       h->split_built = true;
     } else {

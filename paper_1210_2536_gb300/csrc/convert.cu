@@ -26,9 +26,9 @@ template <> struct Bits<2> { typedef unsigned short T; };
 // Row ends of a list: a thread per row marks its last entry, and writes its
 // ordinal for the tiles of 256 entries that start in it (a warp together where
 // they are many) and its row for the ordinal.
-template <typename S>
-__global__ void __launch_bounds__(256) row_ends_kernel(const S *__restrict__ start, const long long *__restrict__ ordinal,
-                                                       long long m, RowEnds re) {
+template <bool CSR>
+__global__ void __launch_bounds__(256) row_ends_kernel(const int32_t *__restrict__ rowptr,
+                                                       const long long *__restrict__ scan, long long m, RowEnds re) {
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long r0 = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; r0 < m; r0 += stride) {
@@ -36,9 +36,10 @@ __global__ void __launch_bounds__(256) row_ends_kernel(const S *__restrict__ sta
     long long t0 = 0, t1 = 0;  // the tiles that start in row r
     int ord = 0;
     if (r < m) {
-      const long long s = start[r], e = start[r + 1];
+      const long long s = CSR ? rowptr[r] : (long long)(unsigned)scan[r];
+      const long long e = CSR ? rowptr[r + 1] : (long long)(unsigned)scan[r + 1];
       if (s < e) {
-        ord = ordinal ? (int)ordinal[r] : (int)r;
+        ord = scan ? (int)(scan[r] >> 32) : (int)r;
         atomicOr(&re.ends[(e - 1) >> 5], 1u << ((e - 1) & 31));
         if (re.row) re.row[ord] = (int32_t)r;
         t0 = (s + 255) >> 8;
@@ -81,7 +82,7 @@ __global__ void empty_rows_kernel(const int32_t *__restrict__ rowptr, long long 
 __global__ void nonempty_rows_kernel(const int32_t *__restrict__ rowptr, long long m, long long *__restrict__ flag) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
        i += (long long)gridDim.x * blockDim.x)
-    flag[i] = rowptr[i + 1] > rowptr[i];
+    flag[i] = (long long)(rowptr[i + 1] > rowptr[i]) << 32;
 }
 
 // ELL: thread per row (and per pad row up to P).
@@ -154,12 +155,12 @@ int grid_for(long long work, int block, int max_blocks) {
 
 size_t row_ends_words(int64_t n) { return (size_t)((n + 255) / 256 * 8); }
 
-cudaError_t launch_row_ends(const RowEnds &re, int64_t m, const int32_t *start32, const long long *start64,
-                            const long long *ordinal, cudaStream_t s) {
+cudaError_t launch_row_ends(const RowEnds &re, int64_t m, const int32_t *rowptr, const long long *scan,
+                            cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   const int g = grid_for(m, 256, 152 * 16);
-  if (start32) row_ends_kernel<<<g, 256, 0, s>>>(start32, ordinal, m, re);
-  else row_ends_kernel<<<g, 256, 0, s>>>(start64, ordinal, m, re);
+  if (rowptr) row_ends_kernel<true><<<g, 256, 0, s>>>(rowptr, scan, m, re);
+  else row_ends_kernel<false><<<g, 256, 0, s>>>(rowptr, scan, m, re);
   return cudaGetLastError();
 }
 

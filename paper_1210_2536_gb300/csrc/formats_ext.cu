@@ -123,36 +123,48 @@ __global__ void scan_tiles(const long long *__restrict__ in, long long n, const 
 }
 
 // ---------------------------------------------------------------------------
+// Lists of entries in row order (HYB's tail, SPLIT's short rows): a row with
+// entries counts 2^32 plus their number, so that one scan gives every row both
+// its ordinal among those rows (high word) and its first entry's place (low).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ long long list_count(long long entries) { return (1ll << 32) + entries; }
+
+// The columns and values of a list's n entries, a warp per tile of 256: entry k
+// of the list is entry rowptr[row] + skip + (k - first[row]) of the matrix.  A
+// thread per row copied rows of up to 10^4 entries alone (SPLIT of the 2e6-row
+// power-law matrix, FP32: 632 us of tuning after the features, now 331).
+template <typename B>
+__global__ void __launch_bounds__(256) list_copy_kernel(RowEnds re, long long n, const int32_t *__restrict__ rowptr,
+                                                        const long long *__restrict__ scan, long long skip,
+                                                        const int32_t *__restrict__ col, const B *__restrict__ val,
+                                                        int32_t *__restrict__ ocol, B *__restrict__ oval) {
+  const int lane = threadIdx.x & 31;
+  const long long tile = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (tile * 256 >= n) return;
+  int ord = re.ord[tile];
+#pragma unroll 4
+  for (int w = 0; w < 8; ++w) {
+    const long long k = tile * 256 + w * 32 + lane;
+    const unsigned ends = re.ends[tile * 8 + w];
+    const int o = ord + __popc(ends & ((1u << lane) - 1u));
+    if (k < n) {
+      const int r = re.row[o];
+      const long long src = rowptr[r] + skip + k - (long long)(unsigned)scan[r];
+      ocol[k] = __ldcs(col + src);
+      oval[k] = val[src];
+    }
+    ord += __popc(ends);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // HYB
 // ---------------------------------------------------------------------------
 __global__ void hyb_tail_counts(const int32_t *__restrict__ rowptr, long long m, long long K,
                                 long long *__restrict__ cnt) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
     const long long rd = rowptr[i + 1] - rowptr[i];
-    cnt[i] = rd > K ? rd - K : 0;
-  }
-}
-
-template <typename B>
-__global__ void to_hyb_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                              const B *__restrict__ val, long long m, long long P, long long K,
-                              const long long *__restrict__ off, int32_t *__restrict__ ecol, B *__restrict__ eval,
-                              int32_t *__restrict__ ccol, B *__restrict__ cval) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
-    long long s = 0, rd = 0;
-    if (i < m) { s = rowptr[i]; rd = rowptr[i + 1] - s; }
-    for (long long q = 0; q < K; ++q) {
-      const long long pos = q * P + i;
-      const bool on = q < rd;
-      ecol[pos] = on ? col[s + q] : -1;
-      eval[pos] = on ? val[s + q] : (B)0;
-    }
-    if (i < m)
-      for (long long q = K; q < rd; ++q) {
-        const long long o = off[i] + q - K;
-        ccol[o] = col[s + q];
-        cval[o] = val[s + q];
-      }
+    cnt[i] = rd > K ? list_count(rd - K) : 0;
   }
 }
 
@@ -237,73 +249,85 @@ __global__ void to_sell_kernel(const int32_t *__restrict__ rowptr, const int32_t
 // ---------------------------------------------------------------------------
 // BCSR
 // ---------------------------------------------------------------------------
-// Thread per block row: a merge of its (up to) b sorted rows, counting the
-// distinct block columns.
+// BS lanes per block row, lane r on row r of it: the lanes step through the
+// distinct block columns together, the smallest next one found by shuffles.  In
+// the fill a lane collects its row of the block in registers and the BS lanes
+// write the whole block contiguously, zeros included.  A thread per block row
+// that zeroed the block and then scattered into it took 184 us on the 8x8
+// blocks of 1e6 rows in FP32 (23 now) and its three counts 111 (44).
+// Groups of a warp that are done keep stepping until the last one is.
+constexpr unsigned BCSR_DONE = UINT_MAX;
+
 template <int BS>
-__global__ void bcsr_count_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, long long m,
-                                  long long mb, long long *__restrict__ cnt) {
-  for (long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x; I < mb; I += (long long)gridDim.x * blockDim.x) {
-    int p[BS], e[BS];
+__device__ __forceinline__ unsigned next_block_column(const int32_t *__restrict__ col, int p, int e) {
+  unsigned j = p < e ? (unsigned)__ldg(col + p) / BS : BCSR_DONE;
 #pragma unroll
-    for (int r = 0; r < BS; ++r) {
-      const long long i = I * BS + r;
-      p[r] = i < m ? rowptr[i] : 0;
-      e[r] = i < m ? rowptr[i + 1] : 0;
-    }
+  for (int o = BS / 2; o > 0; o >>= 1) j = min(j, __shfl_xor_sync(FULL, j, o));
+  return j;
+}
+
+template <int BS>
+__global__ void __launch_bounds__(256) bcsr_count_kernel(const int32_t *__restrict__ rowptr,
+                                                         const int32_t *__restrict__ col, long long m, long long mb,
+                                                         long long *__restrict__ cnt) {
+  const long long stride = (long long)gridDim.x * blockDim.x / BS;
+  const int lane = threadIdx.x & 31, r = lane % BS;
+  for (long long I0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x - lane) / BS; I0 < mb; I0 += stride) {
+    const long long I = I0 + lane / BS, i = I * BS + r;
+    int p = i < m ? rowptr[i] : 0;
+    const int e = i < m ? rowptr[i + 1] : 0;
     long long c = 0;
-    while (true) {
-      unsigned jmin = UINT_MAX;
+    for (;;) {
+      const unsigned j = next_block_column<BS>(col, p, e);
+      if (__all_sync(FULL, j == BCSR_DONE)) break;
+      if (j != BCSR_DONE) ++c;
 #pragma unroll
-      for (int r = 0; r < BS; ++r)
-        if (p[r] < e[r]) jmin = min(jmin, (unsigned)col[p[r]] / BS);
-      if (jmin == UINT_MAX) break;
-      ++c;
-#pragma unroll
-      for (int r = 0; r < BS; ++r)
-        while (p[r] < e[r] && (unsigned)col[p[r]] / BS == jmin) ++p[r];
+      for (int k = 0; k < BS; ++k)
+        if (p < e && (unsigned)__ldg(col + p) / BS == j) ++p;
     }
-    cnt[I] = c;
+    if (r == 0 && I < mb) cnt[I] = c;
   }
 }
 
 template <int BS, typename B>
-__global__ void to_bcsr_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                               const B *__restrict__ val, long long m, long long mb, const long long *__restrict__ brp,
-                               int32_t *__restrict__ browptr, int32_t *__restrict__ bcol, B *__restrict__ bval) {
-  for (long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x; I < mb; I += (long long)gridDim.x * blockDim.x) {
-    const long long k0 = brp[I];
-    browptr[I] = (int32_t)k0;
-    if (I == mb - 1) browptr[mb] = (int32_t)brp[mb];
-    int p[BS], e[BS];
+__global__ void __launch_bounds__(256) to_bcsr_kernel(const int32_t *__restrict__ rowptr,
+                                                      const int32_t *__restrict__ col, const B *__restrict__ val,
+                                                      long long m, long long mb, const long long *__restrict__ brp,
+                                                      int32_t *__restrict__ browptr, int32_t *__restrict__ bcol,
+                                                      B *__restrict__ bval) {
+  constexpr int BYTES = BS * (int)sizeof(B), PIECE = BYTES < 16 ? BYTES : 16;
+  const long long stride = (long long)gridDim.x * blockDim.x / BS;
+  const int lane = threadIdx.x & 31, r = lane % BS;
+  for (long long I0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x - lane) / BS; I0 < mb; I0 += stride) {
+    const long long I = I0 + lane / BS, i = I * BS + r;
+    int p = i < m ? rowptr[i] : 0;
+    const int e = i < m ? rowptr[i + 1] : 0;
+    long long k = I < mb ? brp[I] : 0;
+    if (r == 0 && I < mb) browptr[I] = (int32_t)k;
+    if (r == 0 && I == mb - 1) browptr[mb] = (int32_t)brp[mb];
+    for (;;) {
+      const unsigned j = next_block_column<BS>(col, p, e);
+      if (__all_sync(FULL, j == BCSR_DONE)) break;
+      if (j == BCSR_DONE) continue;
+      alignas(16) B v[BS];
 #pragma unroll
-    for (int r = 0; r < BS; ++r) {
-      const long long i = I * BS + r;
-      p[r] = i < m ? rowptr[i] : 0;
-      e[r] = i < m ? rowptr[i + 1] : 0;
-    }
-    long long k = k0;
-    while (true) {  // the block columns, ascending; their blocks zeroed
-      unsigned jmin = UINT_MAX;
-#pragma unroll
-      for (int r = 0; r < BS; ++r)
-        if (p[r] < e[r]) jmin = min(jmin, (unsigned)col[p[r]] / BS);
-      if (jmin == UINT_MAX) break;
-      bcol[k] = (int32_t)jmin;
-      for (int q = 0; q < BS * BS; ++q) bval[k * BS * BS + q] = (B)0;
-      ++k;
-#pragma unroll
-      for (int r = 0; r < BS; ++r)
-        while (p[r] < e[r] && (unsigned)col[p[r]] / BS == jmin) ++p[r];
-    }
-    for (int r = 0; r < BS; ++r) {  // scatter each row's entries into its blocks
-      const long long i = I * BS + r;
-      if (i >= m) break;
-      long long kb = k0;
-      for (long long q = rowptr[i]; q < rowptr[i + 1]; ++q) {
-        const int J = col[q] / BS;
-        while (bcol[kb] < J) ++kb;
-        bval[kb * BS * BS + r * BS + (col[q] - J * BS)] = val[q];
+      for (int c = 0; c < BS; ++c) {
+        v[c] = (B)0;
+        if (p < e && (unsigned)__ldg(col + p) == j * BS + c) {
+          v[c] = __ldg(val + p);
+          ++p;
+        }
       }
+      char *out = reinterpret_cast<char *>(bval + (k * BS + r) * BS);
+#pragma unroll
+      for (int q = 0; q < BYTES; q += PIECE) {
+        const char *in = reinterpret_cast<const char *>(v) + q;
+        if constexpr (PIECE == 16) *reinterpret_cast<uint4 *>(out + q) = *reinterpret_cast<const uint4 *>(in);
+        else if constexpr (PIECE == 8) *reinterpret_cast<uint2 *>(out + q) = *reinterpret_cast<const uint2 *>(in);
+        else *reinterpret_cast<unsigned *>(out + q) = *reinterpret_cast<const unsigned *>(in);
+      }
+      if (r == 0) bcol[k] = (int32_t)j;
+      ++k;
     }
   }
 }
@@ -312,48 +336,36 @@ __global__ void to_bcsr_kernel(const int32_t *__restrict__ rowptr, const int32_t
 // SPLIT: per-row counts, then each row's entries to their place
 // ---------------------------------------------------------------------------
 __global__ void split_counts_kernel(const int32_t *__restrict__ rowptr, long long m, long long *__restrict__ cl,
-                                    long long *__restrict__ cc, long long *__restrict__ cs,
-                                    long long *__restrict__ ce) {
+                                    long long *__restrict__ cs, long long *__restrict__ ce) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
     const long long rd = rowptr[i + 1] - rowptr[i];
-    const bool lng = rd >= SPLIT_L;
-    cl[i] = lng;
-    cc[i] = lng ? (rd + SPLIT_CK - 1) / SPLIT_CK : 0;
-    cs[i] = (!lng && rd > 0) ? rd : 0;
+    cl[i] = rd >= SPLIT_L ? list_count((rd + SPLIT_CK - 1) / SPLIT_CK) : 0;
+    cs[i] = rd < SPLIT_L && rd > 0 ? list_count(rd) : 0;
     ce[i] = rd == 0;
   }
 }
 
-template <typename B>
-__global__ void split_fill_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                                  const B *__restrict__ val, long long m, const long long *__restrict__ pl,
-                                  const long long *__restrict__ pc, const long long *__restrict__ ps,
+// Long rows' chunks and the empty rows; the short rows' entries are a list.
+__global__ void split_fill_kernel(const int32_t *__restrict__ rowptr, long long m, const long long *__restrict__ pl,
                                   const long long *__restrict__ pe, int32_t *__restrict__ lrows,
                                   int32_t *__restrict__ lchunk, int32_t *__restrict__ crow, int32_t *__restrict__ cstart,
-                                  int32_t *__restrict__ cend, int32_t *__restrict__ scol,
-                                  B *__restrict__ sval, int32_t *__restrict__ empty) {
+                                  int32_t *__restrict__ cend, int32_t *__restrict__ empty) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
     const long long s0 = rowptr[i], e0 = rowptr[i + 1], rd = e0 - s0;
     if (rd == 0) {
       empty[pe[i]] = (int32_t)i;
     } else if (rd >= SPLIT_L) {
-      const long long l = pl[i];
+      const long long l = pl[i] >> 32;
+      long long c = (unsigned)pl[i];
       lrows[l] = (int32_t)i;
-      lchunk[l] = (int32_t)pc[i];
-      long long c = pc[i];
+      lchunk[l] = (int32_t)c;
       for (long long k = s0; k < e0; k += SPLIT_CK, ++c) {
         crow[c] = (int32_t)i;
         cstart[c] = (int32_t)k;
         cend[c] = (int32_t)(k + SPLIT_CK < e0 ? k + SPLIT_CK : e0);
       }
-    } else {
-      long long o = ps[i];
-      for (long long k = s0; k < e0; ++k, ++o) {
-        scol[o] = col[k];
-        sval[o] = val[k];
-      }
     }
-    if (i == 0) lchunk[pl[m]] = (int32_t)pc[m];  // one past the last long row
+    if (i == 0) lchunk[pl[m] >> 32] = (int32_t)(unsigned)pl[m];  // one past the last long row
   }
 }
 
@@ -569,35 +581,24 @@ cudaError_t exclusive_scan(const long long *in, long long n, long long *out, cud
   return e;
 }
 
-__global__ void nonzero_kernel(const long long *__restrict__ count, long long m, long long *__restrict__ flag) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x)
-    flag[i] = count[i] > 0;
-}
-
-cudaError_t launch_nonzero(const long long *count, int64_t m, long long *flag, cudaStream_t s) {
-  if (m <= 0) return cudaSuccess;
-  nonzero_kernel<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(count, m, flag);
+cudaError_t launch_list_copy(const smat_s *h, const RowEnds &re, int64_t n, const long long *scan, int64_t skip,
+                             int32_t *ocol, void *oval, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const unsigned g = (unsigned)((n + 2047) / 2048);
+  switch (h->esz) {
+    case 8: list_copy_kernel<<<g, 256, 0, s>>>(re, n, h->rowptr, scan, skip, h->colidx, (const Raw<8>::T *)h->val, ocol,
+                                                (Raw<8>::T *)oval); break;
+    case 4: list_copy_kernel<<<g, 256, 0, s>>>(re, n, h->rowptr, scan, skip, h->colidx, (const Raw<4>::T *)h->val, ocol,
+                                                (Raw<4>::T *)oval); break;
+    default: list_copy_kernel<<<g, 256, 0, s>>>(re, n, h->rowptr, scan, skip, h->colidx, (const Raw<2>::T *)h->val, ocol,
+                                                 (Raw<2>::T *)oval); break;
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_hyb_tail_counts(const smat_s *h, int64_t K, long long *cnt, cudaStream_t s) {
   if (h->m <= 0) return cudaSuccess;
   hyb_tail_counts<<<grid_for(h->m, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, K, cnt);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_to_hyb(const smat_s *h, int64_t K, const long long *off, int32_t *ecol, void *eval,
-                          int32_t *ccol, void *cval, cudaStream_t s) {
-  if (h->P <= 0) return cudaSuccess;
-  const int g = grid_for(h->P, 256, 152 * 16);
-  switch (h->esz) {
-    case 8: to_hyb_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<8>::T *)h->val, h->m, h->P, K, off, ecol,
-                                              (Raw<8>::T *)eval, ccol, (Raw<8>::T *)cval); break;
-    case 4: to_hyb_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<4>::T *)h->val, h->m, h->P, K, off, ecol,
-                                              (Raw<4>::T *)eval, ccol, (Raw<4>::T *)cval); break;
-    default: to_hyb_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<2>::T *)h->val, h->m, h->P, K, off, ecol,
-                                               (Raw<2>::T *)eval, ccol, (Raw<2>::T *)cval); break;
-  }
   return cudaGetLastError();
 }
 
@@ -629,11 +630,11 @@ cudaError_t launch_to_sell(const smat_s *h, cudaStream_t s) {
 cudaError_t launch_bcsr_count(const smat_s *h, int b, long long *cnt, cudaStream_t s) {
   const long long mb = (h->m + b - 1) / b;
   if (mb <= 0) return cudaSuccess;
-  const int g = grid_for(mb, 128, 152 * 32);
+  const int g = grid_for(mb * b, 256, 152 * 16);
   switch (b) {
-    case 2: bcsr_count_kernel<2><<<g, 128, 0, s>>>(h->rowptr, h->colidx, h->m, mb, cnt); break;
-    case 4: bcsr_count_kernel<4><<<g, 128, 0, s>>>(h->rowptr, h->colidx, h->m, mb, cnt); break;
-    default: bcsr_count_kernel<8><<<g, 128, 0, s>>>(h->rowptr, h->colidx, h->m, mb, cnt); break;
+    case 2: bcsr_count_kernel<2><<<g, 256, 0, s>>>(h->rowptr, h->colidx, h->m, mb, cnt); break;
+    case 4: bcsr_count_kernel<4><<<g, 256, 0, s>>>(h->rowptr, h->colidx, h->m, mb, cnt); break;
+    default: bcsr_count_kernel<8><<<g, 256, 0, s>>>(h->rowptr, h->colidx, h->m, mb, cnt); break;
   }
   return cudaGetLastError();
 }
@@ -641,13 +642,13 @@ cudaError_t launch_bcsr_count(const smat_s *h, int b, long long *cnt, cudaStream
 template <int BS>
 static cudaError_t to_bcsr_b(const smat_s *h, const long long *brp, cudaStream_t s) {
   const long long mb = h->bcsr_mb;
-  const int g = grid_for(mb, 128, 152 * 32);
+  const int g = grid_for(mb * BS, 256, 152 * 16);
   switch (h->esz) {
-    case 8: to_bcsr_kernel<BS><<<g, 128, 0, s>>>(h->rowptr, h->colidx, (const Raw<8>::T *)h->val, h->m, mb, brp,
+    case 8: to_bcsr_kernel<BS><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<8>::T *)h->val, h->m, mb, brp,
                                                    h->bcsr_rowptr, h->bcsr_col, (Raw<8>::T *)h->bcsr_val); break;
-    case 4: to_bcsr_kernel<BS><<<g, 128, 0, s>>>(h->rowptr, h->colidx, (const Raw<4>::T *)h->val, h->m, mb, brp,
+    case 4: to_bcsr_kernel<BS><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<4>::T *)h->val, h->m, mb, brp,
                                                    h->bcsr_rowptr, h->bcsr_col, (Raw<4>::T *)h->bcsr_val); break;
-    default: to_bcsr_kernel<BS><<<g, 128, 0, s>>>(h->rowptr, h->colidx, (const Raw<2>::T *)h->val, h->m, mb, brp,
+    default: to_bcsr_kernel<BS><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<2>::T *)h->val, h->m, mb, brp,
                                                     h->bcsr_rowptr, h->bcsr_col, (Raw<2>::T *)h->bcsr_val); break;
   }
   return cudaGetLastError();
@@ -673,31 +674,17 @@ cudaError_t launch_bcsr_uniform(const smat_s *h, long long c, int *flag, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_counts(const smat_s *h, long long *cl, long long *cc, long long *cs, long long *ce,
-                                cudaStream_t s) {
+cudaError_t launch_split_counts(const smat_s *h, long long *cl, long long *cs, long long *ce, cudaStream_t s) {
   if (h->m <= 0) return cudaSuccess;
-  split_counts_kernel<<<grid_for(h->m, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, cl, cc, cs, ce);
+  split_counts_kernel<<<grid_for(h->m, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, cl, cs, ce);
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_fill(const smat_s *h, const long long *pl, const long long *pc, const long long *ps,
-                              const long long *pe, cudaStream_t s) {
+cudaError_t launch_split_fill(const smat_s *h, const long long *pl, const long long *pe, cudaStream_t s) {
   if (h->m <= 0) return cudaSuccess;
-  const int g = grid_for(h->m, 256, 152 * 16);
-  switch (h->esz) {
-    case 8: split_fill_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<8>::T *)h->val, h->m, pl, pc, ps, pe,
-                                                  h->split_lrows, h->split_lchunk, h->split_crow, h->split_cstart,
-                                                  h->split_cend, h->split_scol,
-                                                  (Raw<8>::T *)h->split_sval, h->split_empty); break;
-    case 4: split_fill_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<4>::T *)h->val, h->m, pl, pc, ps, pe,
-                                                  h->split_lrows, h->split_lchunk, h->split_crow, h->split_cstart,
-                                                  h->split_cend, h->split_scol,
-                                                  (Raw<4>::T *)h->split_sval, h->split_empty); break;
-    default: split_fill_kernel<<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const Raw<2>::T *)h->val, h->m, pl, pc, ps, pe,
-                                                   h->split_lrows, h->split_lchunk, h->split_crow, h->split_cstart,
-                                                   h->split_cend, h->split_scol,
-                                                   (Raw<2>::T *)h->split_sval, h->split_empty); break;
-  }
+  split_fill_kernel<<<grid_for(h->m, 256, 152 * 16), 256, 0, s>>>(h->rowptr, h->m, pl, pe, h->split_lrows,
+                                                                   h->split_lchunk, h->split_crow, h->split_cstart,
+                                                                   h->split_cend, h->split_empty);
   return cudaGetLastError();
 }
 

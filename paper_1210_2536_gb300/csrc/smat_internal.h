@@ -199,16 +199,21 @@ cudaError_t launch_diag_reduce(const int *d_diag_cnt, int64_t m, int64_t n, int 
                                int tau_den, unsigned long long *d_counts, int32_t *d_offsets,
                                int64_t offsets_cap, cudaStream_t s);
 
-// Row ends (convert.cu).  List entries of row r: start[r] .. start[r + 1]
-// (32-bit rowptr or 64-bit scan), none for the rows without any; ordinal[r] =
-// rows with entries before r (nullptr: r).  launch_row_ends fills a zeroed
-// RowEnds; launch_expand_rows writes the row of each of the n entries.
+// Row ends (convert.cu) of a list of entries.  scan[0..m]: the exclusive scan of
+// 2^32 + entries over the rows with entries in the list, 0 over the others, so
+// that row r's entries start at its low word and its ordinal is its high word.
+// With rowptr the entries are the matrix's and scan only numbers the rows
+// (nullptr: no row is empty).  launch_row_ends fills a zeroed RowEnds;
+// launch_expand_rows writes the row of each of the n entries; launch_list_copy
+// copies their columns and values, `skip` entries into each row.
 size_t row_ends_words(int64_t n);
-cudaError_t launch_row_ends(const RowEnds &re, int64_t m, const int32_t *start32, const long long *start64,
-                            const long long *ordinal, cudaStream_t s);
+cudaError_t launch_row_ends(const RowEnds &re, int64_t m, const int32_t *rowptr, const long long *scan,
+                            cudaStream_t s);
+cudaError_t launch_list_copy(const smat_s *h, const RowEnds &re, int64_t n, const long long *scan, int64_t skip,
+                             int32_t *ocol, void *oval, cudaStream_t s);
 cudaError_t launch_expand_rows(const RowEnds &re, int64_t n, int32_t *row, cudaStream_t s);
 cudaError_t launch_empty_rows(const smat_s *h, int32_t *list, int *d_count, cudaStream_t s);
-// flag[r] = 1 when row r has entries.
+// flag[r] = 2^32 when row r has entries, else 0.
 cudaError_t launch_nonempty_rows(const smat_s *h, long long *flag, cudaStream_t s);
 cudaError_t launch_to_ell(const smat_s *h, int64_t K, int32_t *col, void *val, cudaStream_t s);
 cudaError_t launch_to_dia(const smat_s *h, const int32_t *d_off, int64_t nd, void *val,
@@ -218,10 +223,6 @@ cudaError_t launch_to_dia(const smat_s *h, const int32_t *d_off, int64_t nd, voi
 // synchronises `s`.
 cudaError_t exclusive_scan(const long long *in, long long n, long long *out, cudaStream_t s);
 cudaError_t launch_hyb_tail_counts(const smat_s *h, int64_t K, long long *cnt, cudaStream_t s);
-cudaError_t launch_to_hyb(const smat_s *h, int64_t K, const long long *off, int32_t *ecol, void *eval,
-                          int32_t *ccol, void *cval, cudaStream_t s);
-// flag[r] = 1 when count[r] > 0.
-cudaError_t launch_nonzero(const long long *count, int64_t m, long long *flag, cudaStream_t s);
 cudaError_t launch_sell_layout(const smat_s *h, int sigma, int32_t *perm, int32_t *width, long long *cnt,
                                cudaStream_t s);
 cudaError_t launch_to_sell(const smat_s *h, cudaStream_t s);
@@ -230,12 +231,11 @@ cudaError_t launch_bcsr_count(const smat_s *h, int b, long long *cnt, cudaStream
 #define SMAT_SPLIT_L 1024
 #endif
 constexpr int64_t SPLIT_L = SMAT_SPLIT_L, SPLIT_CK = 4096;
-// SPLIT conversion: per-row counts (long flag, chunks, short entries, empty
-// flag) for the scans, then the fill from their exclusive scans.
-cudaError_t launch_split_counts(const smat_s *h, long long *cl, long long *cc, long long *cs, long long *ce,
-                                cudaStream_t s);
-cudaError_t launch_split_fill(const smat_s *h, const long long *pl, const long long *pc, const long long *ps,
-                              const long long *pe, cudaStream_t s);
+// SPLIT conversion: per-row counts for the scans (long rows 2^32 + chunks, short
+// rows 2^32 + entries, empty rows 1), then the long rows' chunks and the list of
+// empty rows.
+cudaError_t launch_split_counts(const smat_s *h, long long *cl, long long *cs, long long *ce, cudaStream_t s);
+cudaError_t launch_split_fill(const smat_s *h, const long long *pl, const long long *pe, cudaStream_t s);
 cudaError_t launch_to_bcsr(const smat_s *h, const long long *brp, cudaStream_t s);
 // Sets *flag (zeroed by the caller) when a block row of the built layout holds
 // a block count other than c.
