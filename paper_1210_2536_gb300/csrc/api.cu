@@ -621,10 +621,17 @@ smat_status_t measure_batch_width(smat_s *h, int variant, cudaStream_t s) {
     }
     return SMAT_OK;
   };
+  float best = 1e30f;
   auto time_it = [&](int u, int lane, float *med) -> smat_status_t {
     for (int w = 0; w < 2; ++w) TRY(launch_spmv_width(h, variant, u, lane, a, x.p, b, y.p, s));
     float wms;
     TRYS(blocks(u, lane, 1, 1, &wms));  // one product alone sizes the repetitions
+    // and one that takes half as long again as the best so far, beyond the
+    // 4 us two single timings may differ by, is not timed further
+    if (wms > 1.5f * best + 0.004f) {
+      *med = wms;
+      return SMAT_OK;
+    }
     const int group = products_per_rep(wms);
     const int nrep = group > 1 ? 3 : 5;   // about as many products as five single ones
     float ms[5];
@@ -633,7 +640,6 @@ smat_status_t measure_batch_width(smat_s *h, int variant, cudaStream_t s) {
     *med = ms[nrep / 2];
     return SMAT_OK;
   };
-  float best = 1e30f;
   int best_u = cand[0];
   for (int c = 0; c < nc; ++c) {
     float med;
