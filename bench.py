@@ -456,7 +456,7 @@ def run_products(args, ctx):
     import torch
     import torch.distributed as dist
     import paper_1210_2536_gb300 as smat
-    from paper_1210_2536_gb300.roofline import algorithmic_bytes, l2_sectors
+    from paper_1210_2536_gb300.roofline import algorithmic_bytes, moved_bytes, moved_sectors
     from paper_1210_2536_gb300.roofline import bound as roof_bound
     from paper_1210_2536_gb300.dist import max_over_ranks, weak_scaling_throughput
     dev, world, rank, select = ctx["dev"], ctx["world"], ctx["rank"], ctx["select"]
@@ -572,7 +572,7 @@ def run_products(args, ctx):
     per = []
     for j, p in enumerate(prods):
         d = statistics.mean(kev[i][j].elapsed_time(kev[i][j + 1]) for i in sampled)
-        byts = algorithmic_bytes(p["f"], p["plan"]["variant"], p["dt"])
+        byts = moved_bytes(p["f"], p["plan"]["variant"], p["dt"])
         csr_bytes = algorithmic_bytes(p["f"], smat.SMAT_V_CSR_SCALAR, p["dt"])
         be = break_even_calls(p["plan"]["tune_ms"], p["csr_ms"], p["pick_ms"])
         per.append({"matrix": p["A"].name, "dtype": p["dt"], "nnz": p["A"].nnz, "variant": p["plan"]["name"],
@@ -603,7 +603,7 @@ def run_products(args, ctx):
     # sector, each streamed 4-byte index 1/8 of one), against the dominant
     # product's own requests: its gathers plus its streamed format bytes
     sector_peak = gather_peak * (1.0 + 4.0 / 32.0)
-    sectors = l2_sectors(dp["f"], dp["plan"]["variant"], dp["dt"])
+    sectors = moved_sectors(dp["f"], dp["plan"]["variant"], dp["dt"])
     sector_frac = sectors / (dom["_d"] / 1e3) / sector_peak
     for r in per:
         r.pop("_d")
@@ -754,7 +754,7 @@ def run_products(args, ctx):
                                    "runs its products one after another on one stream")
                        if args.concurrent else "one stream",
                        "l2": "inputs larger than L2: the step streams "
-                             f"{sum(algorithmic_bytes(p['f'], p['plan']['variant'], p['dt']) for p in prods) / 1e6:.0f}"
+                             f"{sum(moved_bytes(p['f'], p['plan']['variant'], p['dt']) for p in prods) / 1e6:.0f}"
                              " MB and each matrix is evicted by the other products between its launches",
                        "parallelism": f"replicas x{world}"},
             "parity": {"bound": {dt: TOL[dt] for dt in dtypes}, "checked_by": PARITY_TESTS[args.workload]},
@@ -768,7 +768,7 @@ def run_products(args, ctx):
                          "gather_peak_gps": round(gather_peak / 1e9, 1), "gather_frac": round(gather_frac, 4),
                          "l2_sectors_per_launch": sectors, "l2_sector_peak_gps": round(sector_peak / 1e9, 1),
                          "l2_sector_frac": round(sector_frac, 4)},
-            "step_hbm_frac": round(sum(algorithmic_bytes(p["f"], p["plan"]["variant"], p["dt"]) for p in prods)
+            "step_hbm_frac": round(sum(moved_bytes(p["f"], p["plan"]["variant"], p["dt"]) for p in prods)
                                    / (ms / K / 1e3) / 1e9 / peak, 4),
             "gpu_launches": launches_per_step * K,
             "clocks": ck,

@@ -29,7 +29,7 @@
  * Thread safety: calls on different handles are independent.  Products
  * (smat_spmv, smat_spmv_variant) on one handle may run concurrently from
  * different streams and host threads: the kernels that carry partial sums
- * between CTAs (merge-path, COO, HYB, SPLIT) use the handle's own scratch on
+ * between CTAs (CSR_MERGE, COO, HYB, SPLIT) use the handle's own scratch on
  * the first stream that runs products on it and scratch of their own on every
  * further stream, allocated on that stream's first product (so a stream that
  * is capturing a CUDA graph must have run a product on the handle before, or
@@ -299,8 +299,8 @@ smat_status_t smat_spmv_host(smat_handle_t h, const void *alpha, const void *x_h
 smat_status_t smat_variant_bytes(smat_handle_t h, smat_variant_t v, double *bytes);
 
 /* Number of kernel launches one product through variant v issues on this
- * handle (merge-path and COO add a carry fix-up launch when they span more
- * than one tile; COO adds one for empty rows).  Writes 0 for v not built. */
+ * handle (CSR_MERGE and COO add a carry fix-up launch when they span more
+ * than one tile, and one for empty rows).  Writes 0 for v not built. */
 smat_status_t smat_spmv_launches(smat_handle_t h, smat_variant_t v, int32_t *launches);
 
 /* The same host-buffer product without the final synchronisation: the copy
@@ -504,7 +504,7 @@ typedef struct {
                            kernels on side branches of the graph, beside the
                            persistent kernels: 0 none, 1 the members whose
                            plan has no batch kind (SPLIT, COO, HYB, BCSR,
-                           merge-path), 2 all; -1 (default) times 0, 1 (when
+                           CSR_MERGE), 2 all; -1 (default) times 0, 1 (when
                            there are members of both sorts) and, in AUTO
                            mode, 2, and keeps the fastest                     */
 } smat_batch_opts_t;
@@ -526,7 +526,7 @@ void smat_batch_opts_default(smat_batch_opts_t *opts);
 
 /* Group `count` handles of one storage dtype.  The handles stay owned by the
  * caller and must outlive the batch; tune each first (each keeps its plan's
- * format: CSR kernels map to 1/4/8/32 lanes per row, merge-path and COO plans
+ * format: CSR kernels map to 1/4/8/32 lanes per row, CSR_MERGE and COO plans
  * to the fastest measured CSR row kernel, ELL and DIA stay ELL and DIA). */
 smat_status_t smat_batch_create(smat_batch_t *out, const smat_handle_t *hs, int32_t count);
 

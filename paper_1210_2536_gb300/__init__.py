@@ -373,7 +373,7 @@ def smat_mlp_adam(p_ptr, g_ptr, m_ptr, v_ptr, n, t, lr, b1, b2, eps, stream=0):
 
 def smat_spmv_csr_merge_noalloc(m, n, nnz, rowptr_ptr, colidx_ptr, vals_ptr, dtype, alpha_ptr, x_ptr, beta_ptr,
                                 y_ptr, stream=0):
-    """Merge-path CSR product with no allocation (see include/smat.h)."""
+    """CSR product over an even split of the entries, with no allocation (see include/smat.h)."""
     return lib().smat_spmv_csr_merge_noalloc(m, n, nnz, rowptr_ptr, colidx_ptr, vals_ptr, dtype, alpha_ptr, x_ptr,
                                              beta_ptr, y_ptr, stream)
 

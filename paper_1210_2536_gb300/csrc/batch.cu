@@ -239,7 +239,7 @@ int csr_width(const smat_s *h) {
     case SMAT_V_CSR_VEC8: return 8;
     case SMAT_V_CSR_VEC32: return 32;
   }
-  // merge-path / COO plans: the fastest measured CSR row kernel, else by mean row length
+  // CSR_MERGE / COO plans: the fastest measured CSR row kernel, else by mean row length
   int best = -1;
   float bt = 1e30f;
   const int ws[4] = {1, 4, 8, 32};

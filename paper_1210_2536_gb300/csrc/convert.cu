@@ -9,6 +9,8 @@
 //   DIA  val[t * P + i] = a(i, i + off[t]) or +0 where not stored; offsets
 //        ascending.
 //   COO  row[k] for every stored entry, in CSR order (col and val are CSR's).
+//        The products read the row ends as bits (RowEnds); row[k] itself is
+//        written only for an export.
 // Every output element is written exactly once, with coalesced stores, and
 // values are moved as raw bits.
 #include "smat_internal.h"

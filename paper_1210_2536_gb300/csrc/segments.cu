@@ -9,7 +9,7 @@
 // rebased to 0, all N columns), tuned by its own features.  When every
 // segment's plan is a kind the batched kernel runs natively (CSR with 1/4/8/32
 // lanes, ELL, DIA, SELL) the segments run together as one batched launch
-// (batch.cu); otherwise (COO, merge-path, HYB, BCSR) each segment runs its own
+// (batch.cu); otherwise (COO, CSR_MERGE, HYB, BCSR) each segment runs its own
 // plan on a stream of its own, forked from and joined back to the caller's
 // stream, so the segments' kernels overlap.  Both read the shared x and write
 // each segment's slice of y.

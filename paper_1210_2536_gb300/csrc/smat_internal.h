@@ -244,7 +244,7 @@ cudaError_t launch_bcsr_uniform(const smat_s *h, long long c, int *flag, cudaStr
 cudaError_t launch_spmv_ext(const smat_s *h, int variant, const void *alpha, const void *x,
                             const void *beta, void *y, cudaStream_t s);
 
-// Per-product scratch: carries (merge-path, COO, HYB and SPLIT tails) and
+// Per-product scratch: carries (CSR_MERGE, COO, HYB and SPLIT tails) and
 // SPLIT's chunk sums.
 struct Scratch {
   void *carry;

@@ -4,8 +4,9 @@
 // that reuse them (HYB: ELL + COO tail; SPLIT: long rows in CTA chunks and
 // COO tiles of the short rows in one grid, then one closing pass).
 // GPU implementations of CSR follow Bell & Garland (2008, cited by the paper:
-// scalar and vector kernels) and Merrill & Garland (2016: merge-path); COO uses
-// a tiled segmented reduction.
+// scalar and vector kernels); csr_flat.cu holds the CSR kernel that splits the
+// entries evenly.  COO uses a tiled segmented reduction over one bit per entry
+// that marks the row ends, in place of a row index per entry.
 //
 // The kernels stream the format's index and value arrays once with coalesced
 // (ELL, DIA: 16-byte vector or lane-striped) loads, gather x through L1/L2 and
@@ -114,8 +115,10 @@ __global__ void __launch_bounds__(256) csr_vector_kernel(const int32_t *__restri
 // contiguous lanes.  The row open at the tile's end becomes the tile's carry,
 // added by a second kernel.
 //
-// Bound by each SM's gathers in flight.  Before, a row index per entry was
-// loaded (4 of 16 or 12 bytes), every row end was a scattered store, and the
+// Bound by the rate of each SM's L2 sector requests: power-law 2e6 FP64 makes
+// 43.1 M of them in 128.5 us, 1.07 per clock and SM (a kernel of bare gathers
+// and their indices makes 0.96).  Before, a row index per entry was loaded (4
+// of 16 or 12 bytes), every row end was a scattered store, and the
 // scan always took five FP64 steps.  us per product, before and now: power-law
 // 2e6 rows (28.7 M entries) FP64 153.6 -> 130.5, FP32 131.9 -> 111.4; 8e6 rows
 // BF16 520 -> 420; uniform 1e6 FP64 85.4 -> 75.7; 7-point 128^3 FP64 73 -> 50.

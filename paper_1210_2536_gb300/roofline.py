@@ -17,6 +17,12 @@ y written once (plus read when beta != 0):
                                  + 4 empty rows (+ 8 per long row, at most Nchunks: counted as Nchunks)
   every variant                  + s_x N + s_y M (1 + [beta != 0])
 
+COO, the HYB tail and SPLIT's short rows are counted as the format defines
+them, with a 4-byte row index per entry.  The kernels read one bit per entry
+for the row ends and a 4-byte row ordinal per 256 entries instead, and a 4-byte
+row per listed row where rows are left out; ``moved_bytes`` counts that, and
+``bound`` and the bench's sector rate use it.
+
 The HYB / SELL / BCSR / SPLIT sizes come from the built format
 (SpMatrix.features() adds hyb_K, hyb_ncoo, sell_ns, sell_slots, bcsr_b,
 bcsr_nb, split_nc and split_ns once built).
@@ -68,6 +74,33 @@ def algorithmic_bytes(f: dict, variant: int, dtype: str, beta_nonzero: bool = Fa
     return float(mat + sx * n + sx * m * (2 if beta_nonzero else 1))
 
 
+def _row_index_bytes(f: dict, variant: int) -> float:
+    """Bytes the kernels save over the format's row index per entry."""
+    if variant == V_COO:
+        entries, rows = f["nnz"], f["m"] - f["empty_rows"] if f["empty_rows"] else 0
+    elif variant == V_HYB:
+        entries, rows = f["hyb_ncoo"], min(f["hyb_ncoo"], f["m"])
+    elif variant == V_SPLIT:
+        entries, rows = f["split_ns"], min(f["split_ns"], f["m"])
+    else:
+        return 0.0
+    return max(0.0, entries * (4.0 - 1.0 / 8 - 4.0 / 256) - 4.0 * rows)
+
+
+def moved_bytes(f: dict, variant: int, dtype: str, beta_nonzero: bool = False) -> float:
+    """algorithmic_bytes with the row ends the kernels read in place of COO's row indices."""
+    return algorithmic_bytes(f, variant, dtype, beta_nonzero) - _row_index_bytes(f, variant)
+
+
+def moved_sectors(f: dict, variant: int, dtype: str) -> float:
+    """l2_sectors with the row ends in place of COO's row indices (and so
+    without the next-row loads of the FP32 / BF16 tiles)."""
+    n = l2_sectors(f, variant, dtype) - _row_index_bytes(f, variant) / 32.0
+    if variant in (V_COO, V_SPLIT) and dtype != "f64":
+        n -= (f["nnz"] if variant == V_COO else f["split_ns"]) / 8.0
+    return n
+
+
 def flops(f: dict) -> float:
     return 2.0 * f["nnz"]
 
@@ -105,8 +138,9 @@ def l2_sectors(f: dict, variant: int, dtype: str) -> float:
     - y: formats that write rows one at a time from lanes far apart (COO and
       SPLIT tiles, SELL through its row permutation) spend a whole sector per
       row; the others write y in full sectors;
-    - FP32 / BF16 COO and SPLIT tiles also load each thread's next row (one
-      sector per 8 entries; FP64 takes it from the next lane).
+    - a COO with a row index per entry also has each thread of an FP32 / BF16
+      tile load its next row (one sector per 8 entries); ``moved_sectors`` is
+      what the kernels of this library request instead.
     Banded matrices gather x in coalesced runs, so this count holds for
     random-column matrices only."""
     sy = 8 if dtype == "f64" else 4
@@ -134,7 +168,7 @@ def bound(f: dict, variant: int, dtype: str, seconds: float, hbm_gbs: float,
     arithmetic, whichever needs more time at peak; achieved/peak for it.
     fp64_tflops is the measured FP64 roof (smat_measure_fp64_rate x 2);
     without it the derived FP64_PEAK_TFLOPS serves."""
-    byts = algorithmic_bytes(f, variant, dtype)
+    byts = moved_bytes(f, variant, dtype)
     t_hbm = byts / (hbm_gbs * 1e9)
     out = {"bound": "hbm", "achieved": byts / seconds / 1e9, "peak": hbm_gbs, "unit": "GB/s",
            "alg_bytes": byts}

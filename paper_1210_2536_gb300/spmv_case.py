@@ -1,5 +1,5 @@
 """Run one synthetic matrix through chosen SpMV variants and report time,
-GFLOP/s and the fraction of HBM bandwidth each reaches (algorithmic bytes,
+GFLOP/s and the fraction of HBM bandwidth each reaches (bytes moved,
 see roofline.py).  Used for kernel studies and profiler captures:
 
   python -m paper_1210_2536_gb300.spmv_case --matrix stencil3d7:128 --dtype f64 --variant all
@@ -45,7 +45,7 @@ def main():
     import torch
 
     import paper_1210_2536_gb300 as smat
-    from .roofline import algorithmic_bytes
+    from .roofline import moved_bytes
     ap = argparse.ArgumentParser()
     ap.add_argument("--matrix", default="stencil3d7:128")
     ap.add_argument("--dtype", default="f64", choices=["f64", "f32", "bf16"])
@@ -144,7 +144,7 @@ def main():
             t = sorted(s.elapsed_time(e) / group for s, e in ev)
             q = len(t) // 4
             ms = statistics.mean(t[q:len(t) - q])   # mean of the middle half
-            b = algorithmic_bytes(f, v, a.dtype)
+            b = moved_bytes(f, v, a.dtype)
             out["variants"][label] = {"ms": round(ms, 5), "gflops": round(2 * A.nnz / ms / 1e6, 1),
                                       "gbs": round(b / ms / 1e6, 1), "hbm_frac": round(b / ms / 1e6 / peak, 4)}
     print(json.dumps(out))
