@@ -206,7 +206,7 @@ struct smat_batch_s {
   std::vector<const void *> own_x;
   std::vector<void *> own_y;
   std::vector<double> own_a, own_b;
-  static constexpr int OWN_N = 4;
+  static constexpr int OWN_N = 8;
   cudaStream_t cap = nullptr, fork[smat::NKIND - 1] = {}, own_st[OWN_N] = {};
   cudaEvent_t ev_fork = nullptr, ev_join[smat::NKIND - 1] = {}, ev_own[OWN_N] = {};
   cudaGraph_t graph = nullptr;
@@ -343,7 +343,23 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
   b->own_y.assign(n, nullptr);
   b->own_a.assign(n, 1.0);
   b->own_b.assign(n, 0.0);
-  int k_own = 0;
+  // Members that run their own plans go to the side branches largest first,
+  // each to the one with the least work so far.  Eight branches: with four, in
+  // the members' order, a branch of several large products outlived the rest,
+  // and every member's own launches (mode 2) lost to the persistent kernels
+  // beside the others' launches.  us per product, before and now: 29 FP64
+  // matrices on the 128^3 hierarchy 284 -> 267, 27 on 50^3 159 -> 148, 16 FP32
+  // on 96^3 57 -> 55; six branches 270, 152 and 57, sixteen as eight.
+  std::vector<size_t> own_order;
+  for (size_t i = 0; i < n; ++i)
+    if (b->own[i]) own_order.push_back(i);
+  std::stable_sort(own_order.begin(), own_order.end(), [&](size_t a, size_t c) { return b->hs[a]->nnz > b->hs[c]->nnz; });
+  std::vector<int> branch(n, 0);
+  long long load[smat_batch_s::OWN_N] = {};
+  for (size_t i : own_order) {
+    branch[i] = (int)(std::min_element(load, load + smat_batch_s::OWN_N) - load);
+    load[branch[i]] += b->hs[i]->nnz + 400000;  // a launch takes as long as about 400,000 entries
+  }
   for (size_t i = 0; i < n; ++i)
     if (b->own[i]) {
       b->own_x[i] = b->mats[i].x; b->own_y[i] = b->mats[i].y;
@@ -351,8 +367,7 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
       // carries of merge / COO / SPLIT plans: the branch stream's own scratch,
       // allocated now, outside the capture
       Scratch sc{};
-      BTRY(stream_scratch(b->hs[i], b->own_st[k_own % smat_batch_s::OWN_N], &sc, true));
-      ++k_own;
+      BTRY(stream_scratch(b->hs[i], b->own_st[branch[i]], &sc, true));
     }
   dev_free(b->d_tiles);
   b->d_tiles = nullptr;
@@ -393,13 +408,12 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
     err = cudaEventRecord(b->ev_join[k - 1], st[k]);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(b->cap, b->ev_join[k - 1], 0);
   }
-  // the members that run their own plans, round robin on the side branches
-  if (k_own > 0) {
-    const int used = std::min(k_own, smat_batch_s::OWN_N);
+  // the members that run their own plans, on the side branches
+  if (!own_order.empty()) {
+    const int used = (int)std::min(own_order.size(), (size_t)smat_batch_s::OWN_N);
     for (int k = 0; k < used && err == cudaSuccess; ++k) err = cudaStreamWaitEvent(b->own_st[k], b->ev_fork, 0);
-    int j = 0;
-    for (size_t i = 0; i < n && err == cudaSuccess; ++i)
-      if (b->own[i]) err = own_launch(b, i, b->own_st[j++ % smat_batch_s::OWN_N]);
+    for (size_t i : own_order)
+      if (err == cudaSuccess) err = own_launch(b, i, b->own_st[branch[i]]);
     for (int k = 0; k < used && err == cudaSuccess; ++k) {
       err = cudaEventRecord(b->ev_own[k], b->own_st[k]);
       if (err == cudaSuccess) err = cudaStreamWaitEvent(b->cap, b->ev_own[k], 0);

@@ -184,3 +184,29 @@ def test_batch_dia_members(dtype):
     B.close()
     for M in hs:
         M.close()
+
+
+@pytest.mark.parametrize("count", [1, 7, 8, 9, 17])
+def test_batch_own_launches_fill_the_side_branches(count):
+    # fewer members than side branches, as many, one more, and two per branch
+    # and one, COO among them (a scratch of its own per branch), with one
+    # member much larger than the rest
+    mats = [synth.uniform_random(200 + 37 * i, 6.0, i) for i in range(count - 1)] + [synth.powerlaw(20000)]
+    hs = []
+    for i, A in enumerate(mats):
+        M = smat.SpMatrix(A.m, A.n, A.rowptr, A.colidx, A.val, "f64")
+        M.tune("fixed", variant=(smat.SMAT_V_COO, smat.SMAT_V_CSR_VEC4, smat.SMAT_V_CSR_MERGE)[i % 3])
+        hs.append(M)
+    B = smat.Batch(hs)
+    for own in (2, 1, 2):
+        B.tune(trial_reps=3, mode=smat.SMAT_BATCH_GRAPH, own_launches=own)
+        xs = [torch.from_numpy(synth.uniform(own + i, 1, A.n)).to(DEV) for i, A in enumerate(mats)]
+        ys = [torch.full((A.m,), float("nan"), dtype=torch.float64, device=DEV) for A in mats]
+        B.spmv(xs, ys)
+        torch.cuda.synchronize()
+        for i, A in enumerate(mats):
+            ref, scale = reference(A, A.val, xs[i].cpu().numpy(), 1.0, 0.0, None)
+            assert_close_rows(ys[i].cpu().numpy(), ref, scale, TOL["f64"], f"{count} members, own {own}, member {i}")
+    B.close()
+    for M in hs:
+        M.close()
