@@ -354,10 +354,14 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
   for (size_t i = 0; i < n; ++i)
     if (b->own[i]) own_order.push_back(i);
   std::stable_sort(own_order.begin(), own_order.end(), [&](size_t a, size_t c) { return b->hs[a]->nnz > b->hs[c]->nnz; });
+  // Fewer than eight members share four branches: forking and joining a branch
+  // takes longer than the overlap of small products gains (7 FP32 matrices of
+  // a 30^3 hierarchy: 24.6 us on seven branches, 22.6 to 23.6 on four).
+  const int branches = own_order.size() < (size_t)smat_batch_s::OWN_N ? smat_batch_s::OWN_N / 2 : smat_batch_s::OWN_N;
   std::vector<int> branch(n, 0);
   long long load[smat_batch_s::OWN_N] = {};
   for (size_t i : own_order) {
-    branch[i] = (int)(std::min_element(load, load + smat_batch_s::OWN_N) - load);
+    branch[i] = (int)(std::min_element(load, load + branches) - load);
     load[branch[i]] += b->hs[i]->nnz + 400000;  // a launch takes as long as about 400,000 entries
   }
   for (size_t i = 0; i < n; ++i)
@@ -410,7 +414,7 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
   }
   // the members that run their own plans, on the side branches
   if (!own_order.empty()) {
-    const int used = (int)std::min(own_order.size(), (size_t)smat_batch_s::OWN_N);
+    const int used = (int)std::min(own_order.size(), (size_t)branches);
     for (int k = 0; k < used && err == cudaSuccess; ++k) err = cudaStreamWaitEvent(b->own_st[k], b->ev_fork, 0);
     for (size_t i : own_order)
       if (err == cudaSuccess) err = own_launch(b, i, b->own_st[branch[i]]);
