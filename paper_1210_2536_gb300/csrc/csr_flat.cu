@@ -42,8 +42,9 @@ namespace {
 
 constexpr int FLAT_NT = 256, FLAT_WARPS = FLAT_NT / 32;
 constexpr int FLAT_SHIFT = 8, FLAT_CHUNK = 1 << FLAT_SHIFT;  // entries per warp and step
-// A tile that finishes more rows than this leaves the empty ones among them to
-// flat_empty_kernel: one warp writing millions of rows would hold the product.
+// Where a tile finishes more rows than this, flat_empty_kernel writes all of the
+// matrix's empty rows and the tiles none (each is written once: beta must not
+// be applied twice): one warp writing millions of rows would hold the product.
 constexpr int FLAT_MAX_ROWS = 4096;
 
 int grid_for(long long work, int block, int max_blocks) {
@@ -117,14 +118,14 @@ __device__ __forceinline__ int row_past(const int32_t *__restrict__ rowptr, int 
 }
 
 // ALIGNED: col and val take 32-byte (bfloat16: 16-byte) loads; otherwise each
-// entry is loaded by itself.  empty: this kernel writes the empty rows too.
+// entry is loaded by itself.  write_empty: this kernel writes the empty rows too.
 template <typename V, typename T, int MODE, bool ALIGNED>
 __global__ void __launch_bounds__(FLAT_NT) csr_flat_kernel(const int32_t *__restrict__ rowptr,
                                                            const int32_t *__restrict__ col, const V *__restrict__ val,
                                                            const T *__restrict__ x, Epi<T, MODE> ep,
                                                            T *__restrict__ y, long long nnz,
                                                            const int32_t *__restrict__ tile_row, long long ntiles,
-                                                           int chunks, int empty, int32_t *__restrict__ carry_row,
+                                                           int chunks, bool write_empty, int32_t *__restrict__ carry_row,
                                                            T *__restrict__ carry_val) {
   griddep_wait();
   constexpr int IPT = 8;
@@ -139,7 +140,6 @@ __global__ void __launch_bounds__(FLAT_NT) csr_flat_kernel(const int32_t *__rest
   unsigned *end = s_end[w];
   int r = __ldg(tile_row + tile);
   const int rend = __ldg(tile_row + tile + 1);
-  const bool write_empty = empty && rend - r <= FLAT_MAX_ROWS;
   T run = 0;  // what the row open at the end of the last chunk holds
   int last_end = 0;
   for (int ch = 0; ch < chunks; ++ch) {
@@ -249,7 +249,7 @@ cudaError_t flat_mode(const FlatArgs &a, typename Compute<V>::T alpha, const voi
   e = launch_pdl(aligned ? csr_flat_kernel<V, T, MODE, true> : csr_flat_kernel<V, T, MODE, false>,
                  dim3((unsigned)((a.tiles + FLAT_WARPS - 1) / FLAT_WARPS)), dim3(FLAT_NT), 0, s, a.rowptr, a.col,
                  (const V *)a.val, x, ep, y, a.nnz, (const int32_t *)a.tile_row, a.tiles, 1 << a.log2_chunks,
-                 a.rows_pass ? 0 : 1, a.carry_row, (T *)a.carry_val);
+                 !a.rows_pass && !a.empty_pass, a.carry_row, (T *)a.carry_val);
   if (e != cudaSuccess || a.tiles == 1) return e;
   return launch_pdl(carry_kernel<T, MODE>, dim3(grid_for(a.tiles, 256, 152 * 8)), nt, 0, s, (const int32_t *)nullptr,
                     (const int32_t *)a.carry_row, (const T *)a.carry_val, a.tiles, ep, y);

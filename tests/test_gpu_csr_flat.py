@@ -82,6 +82,41 @@ def test_edges(name, A, dtype):
     M.close()
 
 
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("name,A", list(_cases()), ids=[k for k, _ in _cases()])
+def test_every_row_takes_beta_once(name, A, dtype):
+    # beta other than 0 and 1: a row written twice, or not at all, shows.  The
+    # gaps case joins tiles of more than FLAT_MAX_ROWS rows with tiles that
+    # hold short runs of empty rows.
+    vals, vals64 = stored_values(A, dtype)
+    vals = np.ascontiguousarray(vals.view(np.int16) if dtype == "bf16" else vals)
+    np_t = np.float64 if dtype == "f64" else np.float32
+    ct = ctypes.c_double if dtype == "f64" else ctypes.c_float
+    x = synth.uniform(1, 1, A.n).astype(np_t)
+    y0 = synth.uniform(2, 1, A.m).astype(np_t)
+    xd, rp, ci, vv = (torch.from_numpy(t).to(DEV) for t in (x, A.rowptr, A.colidx, vals))
+    M = smat.SpMatrix(A.m, A.n, A.rowptr, A.colidx, vals, dtype)
+    N = smat.SpMatrix(A.m, A.n, A.rowptr, A.colidx, vals, dtype)
+    N.tune("fixed", variant=smat.SMAT_V_CSR_MERGE)
+    for alpha, beta in ((2.0, -0.5), (1.0, 2.0), (1.5, -0.75)):
+        ref, scale = reference(A, vals64, x, alpha, beta, y0)
+        y = torch.from_numpy(y0.copy()).to(DEV)
+        M.spmv(xd, y, alpha, beta, variant=smat.SMAT_V_CSR_MERGE)
+        assert_close_rows(y.cpu().numpy().astype(np.float64), ref, scale, TOL[dtype], f"{name} {alpha} {beta}")
+        y = torch.from_numpy(y0.copy()).to(DEV)
+        N.spmv(xd, y, alpha, beta)
+        assert_close_rows(y.cpu().numpy().astype(np.float64), ref, scale, TOL[dtype], f"{name} plan {alpha} {beta}")
+        y = torch.from_numpy(y0.copy()).to(DEV)
+        a, b = ct(alpha), ct(beta)
+        st = smat.smat_spmv_csr_merge_noalloc(A.m, A.n, A.nnz, rp.data_ptr(), ci.data_ptr(), vv.data_ptr(),
+                                              smat.DTYPES[dtype], ctypes.addressof(a), xd.data_ptr(),
+                                              ctypes.addressof(b), y.data_ptr(),
+                                              torch.cuda.current_stream().cuda_stream)
+        assert st == smat.SMAT_OK
+        assert_close_rows(y.cpu().numpy().astype(np.float64), ref, scale, TOL[dtype], f"{name} noalloc {alpha} {beta}")
+    M.close(), N.close()
+
+
 def test_noalloc_several_chunks_per_tile():
     # 65536 tiles of one chunk hold 16.8 M entries: this matrix takes two per
     # tile, with rows that cross chunks and tiles

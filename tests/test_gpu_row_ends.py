@@ -72,3 +72,31 @@ def test_products_and_exports(name, dtype):
             assert np.array_equal(got, row[keep])
     assert built >= 1
     M.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("name", list(CASES))
+def test_every_row_takes_beta_once(name, dtype):
+    # beta other than 0 and 1: a row written twice, or not at all, shows
+    A = _rows(CASES[name], 40000, 11)
+    vals, vals64 = stored_values(A, dtype)
+    vals = np.ascontiguousarray(vals.view(np.int16) if dtype == "bf16" else vals)
+    np_t = np.float64 if dtype == "f64" else np.float32
+    M = smat.SpMatrix(A.m, A.n, A.rowptr, A.colidx, vals, dtype)
+    M.tune("fixed", variant=smat.SMAT_V_CSR_SCALAR, keep_formats=1, fill_ratio_max=100000, bytes_cap=1e9)
+    x = synth.uniform(1, 1, A.n).astype(np_t)
+    y0 = synth.uniform(2, 1, A.m).astype(np_t)
+    xd = torch.from_numpy(x).to(DEV)
+    for v, fmt in ((smat.SMAT_V_COO, smat.SMAT_FMT_COO), (smat.SMAT_V_SPLIT, smat.SMAT_FMT_SPLIT),
+                   (smat.SMAT_V_HYB, smat.SMAT_FMT_HYB)):
+        try:
+            M.convert(fmt)
+        except smat.SmatError as e:
+            assert e.status == smat.SMAT_ERR_UNSUPPORTED and v != smat.SMAT_V_COO
+            continue
+        for alpha, beta in ((2.0, -0.5), (1.0, 2.0), (1.5, -0.75)):
+            y = torch.from_numpy(y0.copy()).to(DEV)
+            M.spmv(xd, y, alpha, beta, variant=v)
+            ref, scale = reference(A, vals64, x, alpha, beta, y0)
+            assert_close_rows(y.cpu().numpy().astype(np.float64), ref, scale, TOL[dtype], f"{name} {v} {alpha} {beta}")
+    M.close()
