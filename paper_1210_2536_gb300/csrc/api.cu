@@ -856,6 +856,17 @@ cudaError_t stream_scratch(const smat_s *h, cudaStream_t s, Scratch *out, bool c
   return cudaSuccess;
 }
 
+void release_stream_scratch(const smat_s *h, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(h->scratch_mu);
+  if (h->scratch_owned && h->scratch_owner == s) h->scratch_owned = false;
+  for (size_t i = 0; i < h->more_scratch.size(); ++i)
+    if (h->more_scratch[i].stream == s) {
+      dev_free(h->more_scratch[i].p);
+      h->more_scratch.erase(h->more_scratch.begin() + (long)i);
+      break;
+    }
+}
+
 void free_stream_scratch(smat_s *h) {
   for (auto &e : h->more_scratch) dev_free(e.p);
   h->more_scratch.clear();

@@ -503,6 +503,10 @@ extern "C" smat_status_t smat_cg_mixed(smat_handle_t a64, smat_handle_t a32, con
     if (!chk(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking))) break;
     if (!chk(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming))) break;
     if (!chk(cudaEventRecord(ev, user)) || !chk(cudaStreamWaitEvent(s, ev, 0))) break;
+    // the inner products' carries on s, which cannot be allocated while it
+    // captures: other streams may hold the handle's own
+    Scratch carries;
+    if (needs_scratch(a32, a32->variant) && !chk(stream_scratch(a32, s, &carries))) break;
     if (!chk(cudaMemsetAsync(sc, 0, sizeof(CgScalars), s))) break;
     dot64_kernel<<<gb, CG_NT, 0, s>>>(b, b, n, part64, sc);
     double bb = 0.0;
@@ -570,7 +574,11 @@ extern "C" smat_status_t smat_cg_mixed(smat_handle_t a64, smat_handle_t a32, con
   if (gexec) cudaGraphExecDestroy(gexec);
   if (graph) cudaGraphDestroy(graph);
   if (ev) cudaEventDestroy(ev);
-  if (s) cudaStreamDestroy(s);
+  if (s) {
+    release_stream_scratch(a64, s);
+    release_stream_scratch(a32, s);
+    cudaStreamDestroy(s);
+  }
   inf.relres = nb > 0.0 ? nr / nb : 0.0;
   if (nb > 0.0 && inf.relres <= o.rtol) inf.converged = 1;
   inf.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

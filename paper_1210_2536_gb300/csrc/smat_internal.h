@@ -256,6 +256,11 @@ struct Scratch {
 // uses the handle's buffers without making s their owner.
 cudaError_t stream_scratch(const smat_s *h, cudaStream_t s, Scratch *out, bool claim = true);
 void free_stream_scratch(smat_s *h);
+// Gives back what stream s holds of h's scratch, for a stream that ends: its
+// own buffer is freed, and the handle's buffers may be claimed again.
+void release_stream_scratch(const smat_s *h, cudaStream_t s);
+// Whether a product through `variant` uses scratch.
+bool needs_scratch(const smat_s *h, int variant);
 // CSR split evenly by entries (csr_flat.cu): its tiles, the kernels that fill
 // tile_row[tiles + 1] and set *gaps (zeroed by the caller), and the product.
 long long flat_tiles(long long nnz);

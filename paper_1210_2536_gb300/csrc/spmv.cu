@@ -567,6 +567,10 @@ size_t carry_bytes_needed(const smat_s *h, int variant) {
   return (size_t)((tiles * 4 + 15) / 16) * 16 + (size_t)tiles * tsz;
 }
 
+bool needs_scratch(const smat_s *h, int variant) {
+  return carry_bytes_needed(h, variant) > 0 || variant == SMAT_V_SPLIT;
+}
+
 int spmv_launch_count(const smat_s *h, int variant) {
   if (h->m == 0) return 0;
   if (variant == SMAT_V_CSR_MERGE) {
@@ -625,7 +629,7 @@ cudaError_t launch_spmv(const smat_s *h, int variant, const void *alpha, const v
     variant = SMAT_V_CSR_SCALAR;
   if (variant == SMAT_V_SELL || variant == SMAT_V_BCSR) return launch_spmv_ext(h, variant, alpha, x, beta, y, s);
   Scratch sc{nullptr, nullptr};
-  if (carry_bytes_needed(h, variant) > 0 || variant == SMAT_V_SPLIT) {
+  if (needs_scratch(h, variant)) {
     cudaError_t e = stream_scratch(h, s, &sc, claim);
     if (e != cudaSuccess) return e;
   }

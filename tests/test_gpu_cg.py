@@ -109,3 +109,38 @@ def test_vector_kernel_sizes(n):
     err = np.linalg.norm(xd.cpu().numpy() - x_true) / np.linalg.norm(x_true)
     assert err <= 4e-12, err
     A64.close(), A32.close()
+
+
+def arrow(n):
+    """A symmetric, diagonally dominant matrix with one full row and column."""
+    i = np.arange(1, n)
+    r = np.concatenate([[0], i, np.zeros(n - 1, int), i, i[1:], i[:-1]])
+    c = np.concatenate([[0], i, i, np.zeros(n - 1, int), i[:-1], i[1:]])
+    v = np.concatenate([np.full(n, 4.0), np.full(2 * (n - 1), -1e-3), np.full(2 * (n - 2), -1.0)])
+    o = np.lexsort((c, r))
+    rowptr = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=n))])
+    return synth.CSR(n, n, rowptr.astype(np.int32), c[o].astype(np.int32), v[o])
+
+
+@pytest.mark.parametrize("variant", ["CSR_MERGE", "COO", "HYB", "SPLIT"])
+def test_inner_plans_with_carries_on_a_handle_in_use(variant):
+    # the inner handle's carries belong to the caller's stream already; the
+    # solve's own stream needs some of its own before it captures, and leaves
+    # none behind
+    A = arrow(3000)
+    x_true = synth.uniform(4, 5, A.n)
+    b = oracle.spmv_csr(A.m, A.rowptr, A.colidx, A.val, x_true, threads=8)
+    bd = torch.from_numpy(b).to(DEV)
+    A64, A32 = handles(A, tune=False)
+    for M in (A64, A32):
+        M.tune("fixed", variant=getattr(smat, "SMAT_V_" + variant))
+    x32 = torch.from_numpy(x_true.astype(np.float32)).to(DEV)
+    before = A32.spmv(x32)
+    A64.spmv(bd)
+    for solve in range(3):
+        xd = torch.zeros(A.n, dtype=torch.float64, device=DEV)
+        info = smat.cg_mixed(A64, A32, bd, xd, rtol=1e-11, use_graph=int(solve < 2))
+        assert info["converged"], info
+        assert oracle_relres(A, xd.cpu().numpy(), b) <= 1.1e-11
+    assert torch.equal(A32.spmv(x32), before)
+    A64.close(), A32.close()
