@@ -685,7 +685,10 @@ void smat_test_fail_alloc_after(int32_t k);
  * then give up; the kernel still waits for its own copies before it leaves,
  * counts the timeout (smat_get_wait_timeouts) and returns, leaving the
  * context usable.  The products run meanwhile are invalid.  on = 0 restores
- * normal operation.  For tests of the failure path. */
+ * normal operation.  For tests of the failure path.  The grid barriers of
+ * smat_cg_mixed (n > 32768) are not passed meanwhile either: the first waits
+ * for wait_cycles (0: about two seconds), the following ones briefly, and the
+ * solve returns SMAT_ERR_CUDA with x as it was before the refinement step. */
 void smat_test_stall_pipelines(int32_t on, int64_t wait_cycles);
 
 /* ------------------------------------------------------------------------ */

@@ -33,6 +33,15 @@ constexpr int CG_BLOCKS = 152 * 4;
 // 768 x 4 97.4, 1024 x 3 95.9 with spills, 512 x 8 98.9; 2^21 rows 11.6-13.1).
 constexpr int CV_RESIDENT_NT = 1024, CV_STREAM_NT = 768, CV_U = 3;
 
+// A grid barrier's wait, in SM clocks: about two seconds, and half a millisecond
+// once a barrier of the solve has given up (passing one takes a few us; the
+// streaming passes before it, up to 100 us on 2^24 rows).
+constexpr long long CV_WAIT = 4000000000ll, CV_WAIT_STALLED = 1ll << 20;
+struct GridWait {
+  long long limit;
+  int never;  // test hook: no barrier is passed
+};
+
 // Device-side scalars of one solve.
 struct CgScalars {
   float rho, rho0;
@@ -133,10 +142,13 @@ __global__ void __launch_bounds__(CG_NT) inner_init_kernel(const double *__restr
 }
 
 // One thread of each CTA: waits until every CTA of the grid (all resident: a
-// cooperative launch) has arrived.  The wait is bounded (about two seconds of
-// SM clocks): a grid that gives up sets sc->stalled, which the host reads with
-// the residual, and every CTA still runs to its end.
-__device__ __forceinline__ void grid_arrive_wait(CgScalars *sc) {
+// cooperative launch) has arrived.  The wait is bounded: a grid that gives up
+// sets sc->stalled, which the host reads with the residual, and every CTA still
+// runs to its end, arriving at each barrier.  The iterations queued behind it are
+// invalid too, so from then on a barrier that is not passed soon is left: the
+// host looks only after a chunk, whose every barrier would otherwise wait for
+// the whole limit.
+__device__ __forceinline__ void grid_arrive_wait(CgScalars *sc, const GridWait &wait) {
   __threadfence();
   const unsigned ticket = atomicAdd(&sc->arrived, 1u);
   const unsigned target = ticket - ticket % gridDim.x + gridDim.x;
@@ -144,8 +156,9 @@ __device__ __forceinline__ void grid_arrive_wait(CgScalars *sc) {
   for (;;) {
     unsigned now;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&sc->arrived) : "memory");
-    if ((int)(now - target) >= 0) break;
-    if (clock64() - t0 > 4000000000ll) {
+    if ((int)(now - target) >= 0 && !wait.never) break;
+    const long long waited = clock64() - t0;
+    if (waited > wait.limit || (waited > CV_WAIT_STALLED && *(volatile int *)&sc->stalled)) {
       sc->stalled = 1;
       break;
     }
@@ -165,7 +178,7 @@ __device__ __forceinline__ float warp_total(float v) {
 // them reading (24 K requests for the same lines) a sum over 147 CTAs took
 // 7 us instead of 2.
 template <bool CLUSTER, int NT>
-__device__ __forceinline__ float grid_sum(float v, float *partials, CgScalars *sc) {
+__device__ __forceinline__ float grid_sum(float v, float *partials, CgScalars *sc, const GridWait &wait) {
   __shared__ float sh[NT / 32], total;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   v = warp_total(v);
@@ -178,7 +191,7 @@ __device__ __forceinline__ float grid_sum(float v, float *partials, CgScalars *s
         total = v;
       } else {
         partials[blockIdx.x] = v;
-        if (!CLUSTER) grid_arrive_wait(sc);
+        if (!CLUSTER) grid_arrive_wait(sc, wait);
       }
     }
     __syncwarp();
@@ -236,7 +249,7 @@ __device__ __forceinline__ float sum_of(const float (&a)[CV_U]) {
 template <bool CLUSTER, bool RESIDENT, int NT = RESIDENT ? CV_RESIDENT_NT : CV_STREAM_NT>
 __global__ void __launch_bounds__(NT, 1) cg_vector_kernel(float *__restrict__ p, const float *__restrict__ q,
                                                           float *__restrict__ d, float *__restrict__ res, int n,
-                                                          float *partials, CgScalars *sc) {
+                                                          float *partials, CgScalars *sc, GridWait wait) {
   griddep_wait();
   const float rho = __ldcg(&sc->rho);  // CTA 0 writes the new one after the last sum
   const int n4 = n / 4, step = gridDim.x * NT, first = blockIdx.x * NT + threadIdx.x;
@@ -251,11 +264,11 @@ __global__ void __launch_bounds__(NT, 1) cg_vector_kernel(float *__restrict__ p,
     float4 R = on ? r4[first] : zero;
     const float tp = tail ? p[it] : 0.0f, tq = tail ? q[it] : 0.0f, td = tail ? d[it] : 0.0f;
     float tr = tail ? res[it] : 0.0f;
-    const float pq = grid_sum<CLUSTER, NT>(dot4(P, Q, tp * tq), partials, sc);
+    const float pq = grid_sum<CLUSTER, NT>(dot4(P, Q, tp * tq), partials, sc, wait);
     const float alpha = (pq > 0.0f && rho > 0.0f) ? rho / pq : 0.0f;
     R = fma4(-alpha, Q, R);
     tr = fmaf(-alpha, tq, tr);
-    const float rho1 = grid_sum<CLUSTER, NT>(dot4(R, R, tr * tr), partials + gridDim.x, sc);
+    const float rho1 = grid_sum<CLUSTER, NT>(dot4(R, R, tr * tr), partials + gridDim.x, sc, wait);
     const float beta = rho > 0.0f ? rho1 / rho : 0.0f;
     if (blockIdx.x == 0 && threadIdx.x == 0) sc->rho = rho1;
     if (on) {
@@ -286,7 +299,7 @@ __global__ void __launch_bounds__(NT, 1) cg_vector_kernel(float *__restrict__ p,
     for (int k = 0; k < CV_U; ++k) acc[k] = dot4(a[k], b[k], acc[k]);
   }
   if (tail) acc[0] = fmaf(p[it], q[it], acc[0]);
-  const float pq = grid_sum<CLUSTER, NT>(sum_of(acc), partials, sc);
+  const float pq = grid_sum<CLUSTER, NT>(sum_of(acc), partials, sc, wait);
   const float alpha = (pq > 0.0f && rho > 0.0f) ? rho / pq : 0.0f;
 #pragma unroll
   for (int k = 0; k < CV_U; ++k) acc[k] = 0.0f;
@@ -311,7 +324,7 @@ __global__ void __launch_bounds__(NT, 1) cg_vector_kernel(float *__restrict__ p,
     res[it] = v;
     acc[0] = fmaf(v, v, acc[0]);
   }
-  const float rho1 = grid_sum<CLUSTER, NT>(sum_of(acc), partials + gridDim.x, sc);
+  const float rho1 = grid_sum<CLUSTER, NT>(sum_of(acc), partials + gridDim.x, sc, wait);
   const float beta = rho > 0.0f ? rho1 / rho : 0.0f;
   if (blockIdx.x == 0 && threadIdx.x == 0) sc->rho = rho1;
   for (int t = rounds - 1; t >= 0; --t) {
@@ -385,7 +398,7 @@ VectorShape vector_shape(long long n) {
 }
 
 cudaError_t launch_cg_vector(const VectorShape &v, float *p, const float *q, float *d, float *res, long long n,
-                             float *partials, CgScalars *sc, cudaStream_t s) {
+                             float *partials, CgScalars *sc, const GridWait &wait, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)v.ctas);
   cfg.blockDim = dim3(v.resident ? CV_RESIDENT_NT : CV_STREAM_NT);
@@ -399,13 +412,13 @@ cudaError_t launch_cg_vector(const VectorShape &v, float *p, const float *q, flo
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, cg_vector_kernel<true, true>, p, q, d, res, (int)n, partials, sc);
+    return cudaLaunchKernelEx(&cfg, cg_vector_kernel<true, true>, p, q, d, res, (int)n, partials, sc, wait);
   }
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, v.resident ? cg_vector_kernel<false, true> : cg_vector_kernel<false, false>, p, q, d,
-                            res, (int)n, partials, sc);
+                            res, (int)n, partials, sc, wait);
 }
 
 struct Workspace {
@@ -470,6 +483,9 @@ extern "C" smat_status_t smat_cg_mixed(smat_handle_t a64, smat_handle_t a32, con
   smat_status_t status = SMAT_OK;
   const int gb = blocks_for(n);
   const VectorShape gv = vector_shape(n);
+  GridWait wait{CV_WAIT, 0};
+  long long stall_cycles = 0;
+  if (stall_waits(&stall_cycles)) wait = {stall_cycles > 0 ? stall_cycles : CV_WAIT, 1};
   const double one = 1.0, mone = -1.0;
   const float onef = 1.0f, zerof = 0.0f;
   double nb = 0.0, nr = 0.0;
@@ -484,7 +500,7 @@ extern "C" smat_status_t smat_cg_mixed(smat_handle_t a64, smat_handle_t a32, con
   };
   auto inner_iteration = [&]() -> bool {
     if (!spmv32()) return false;
-    return chk(launch_cg_vector(gv, p, q, d, res, n, part32, sc, s));
+    return chk(launch_cg_vector(gv, p, q, d, res, n, part32, sc, wait, s));
   };
   auto residual_norm = [&](double *out) -> bool {
     // r = b - A64 x in FP64, then ||r||

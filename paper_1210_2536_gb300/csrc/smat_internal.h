@@ -288,6 +288,9 @@ int dia_staged_kernels();
 bool dia_staged_ok(const smat_s *h, int kernel);
 cudaError_t launch_dia_staged(const smat_s *h, int kernel, const void *alpha, const void *x, const void *beta,
                               void *y, cudaStream_t s, long long wait_limit = 0);
+// Whether the test hook makes bounded waits run out, and after how many cycles
+// (0: the wait's own limit).
+bool stall_waits(long long *cycles);
 // SpMV through one variant; alpha/beta are host scalars of the compute type.
 // claim: as in stream_scratch (false for the tuner's timing products).
 cudaError_t launch_spmv(const smat_s *h, int variant, const void *alpha, const void *x,

@@ -39,7 +39,8 @@ constexpr long long ST_WAIT_CYCLES = 2000000000LL;
 __device__ unsigned long long g_wait_timeouts;
 
 // Test hook (smat_test_stall_pipelines): consumers wait on a barrier that
-// nothing arrives on, for `cycles`, so that the timeout path runs.
+// nothing arrives on, for `cycles`, so that the timeout path runs (and the CG's
+// grid barriers are not passed).
 std::atomic<int> g_stall_on{0};
 std::atomic<long long> g_stall_cycles{0};
 
@@ -262,6 +263,11 @@ cudaError_t launch_dia_staged(const smat_s *h, int kernel, const void *alpha, co
     case SMAT_F32: return dia_staged_typed<float>(cfg, h, g, alpha, x, beta, y, s, wait_limit);
     default: return dia_staged_typed<__nv_bfloat16>(cfg, h, g, alpha, x, beta, y, s, wait_limit);
   }
+}
+
+bool stall_waits(long long *cycles) {
+  *cycles = g_stall_cycles.load();
+  return g_stall_on.load() != 0;
 }
 
 cudaError_t wait_timeouts(unsigned long long *out) {

@@ -1,5 +1,7 @@
 """Mixed-precision CG: FP32/BF16 inner solves, FP64 residual and update.
 The final residual is recomputed on the host by the oracle's FP64 SpMV."""
+import time
+
 import numpy as np
 import pytest
 
@@ -108,6 +110,46 @@ def test_vector_kernel_sizes(n):
     assert info["converged"], info
     err = np.linalg.norm(xd.cpu().numpy() - x_true) / np.linalg.norm(x_true)
     assert err <= 4e-12, err
+    A64.close(), A32.close()
+
+
+def tridiagonal(n):
+    i = np.arange(n)
+    cols = np.stack([i - 1, i, i + 1], 1)
+    ok = (cols >= 0) & (cols < n)
+    val = np.broadcast_to(np.array([-1.0, 4.0, -1.0]), (n, 3))[ok].copy()
+    rowptr = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    return synth.CSR(n, n, rowptr, cols[ok].astype(np.int32), val)
+
+
+@pytest.mark.parametrize("graph", [1, 0])
+@pytest.mark.parametrize("n", [40000, 1400001])
+def test_grid_barriers_that_run_out_end_the_solve(n, graph):
+    # the test hook keeps every grid barrier from being passed (vectors in
+    # registers, and streamed).  The first waits for 6e8 cycles (0.3 s); the
+    # other 39 of the chunk half a millisecond each, 20 ms in all, where they
+    # would take 12 s if each waited for its limit.
+    A = tridiagonal(n)
+    b = oracle.spmv_csr(n, A.rowptr, A.colidx, A.val, synth.uniform(3, 5, n), threads=8)
+    A64, A32 = handles(A, tune=False)
+    bd = torch.from_numpy(b).to(DEV)
+    xd = torch.zeros(n, dtype=torch.float64, device=DEV)
+    opts = dict(rtol=1e-12, check_every=20, use_graph=graph)
+    assert smat.cg_mixed(A64, A32, bd, xd, **opts)["converged"]
+    good = xd.clone()
+    xd.fill_(1.0)
+    smat.lib().smat_test_stall_pipelines(1, 600_000_000)
+    try:
+        t0 = time.monotonic()
+        with pytest.raises(smat.SmatError) as e:
+            smat.cg_mixed(A64, A32, bd, xd, **opts)
+        assert e.value.status == smat.SMAT_ERR_CUDA and time.monotonic() - t0 < 4.0
+    finally:
+        smat.lib().smat_test_stall_pipelines(0, 0)
+    assert bool((xd == 1.0).all())            # no refinement step was taken
+    xd.zero_()
+    assert smat.cg_mixed(A64, A32, bd, xd, **opts)["converged"]
+    assert torch.equal(xd, good)              # the context is usable, the solve reproducible
     A64.close(), A32.close()
 
 
