@@ -14,6 +14,8 @@
 // iterations are replayed from a CUDA graph.  Every sum is taken in a fixed
 // order, so a solve is reproducible.  The host reads the residual only between
 // chunks.
+#include <cuda.h>
+
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -381,14 +383,44 @@ struct VectorShape {
   bool cluster, resident;
 };
 
-VectorShape vector_shape(long long n) {
-  int dev = 0, sms = 1;
+// The device's SMs, and those that the current context may use: a green
+// context holds some of them only, and CTAs beyond its own are never resident
+// together.
+template <typename F>
+F driver_function(const char *name, unsigned version) {
+  void *p = nullptr;
+  cudaDriverEntryPointQueryResult r;
+  if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &r) != cudaSuccess ||
+      r != cudaDriverEntryPointSuccess)
+    p = nullptr;
+  return (F)p;
+}
+
+void count_sms(int *device, int *context) {
+  static const auto current = driver_function<CUresult (*)(CUcontext *)>("cuCtxGetCurrent", 4000);
+  static const auto resource =
+      driver_function<CUresult (*)(CUcontext, CUdevResource *, CUdevResourceType)>("cuCtxGetDevResource", 12040);
+  int dev = 0;
+  *device = 1;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    sms = 1;
+      cudaDeviceGetAttribute(device, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    *device = 1;
+  *context = *device;
+  CUcontext ctx = nullptr;
+  CUdevResource res;
+  if (current && resource && current(&ctx) == CUDA_SUCCESS && ctx &&
+      resource(ctx, &res, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && res.sm.smCount > 0)
+    *context = std::min(*device, (int)res.sm.smCount);
+}
+
+VectorShape vector_shape(long long n) {
+  int device, sms;
+  count_sms(&device, &sms);
   // CTAs of one float4 per thread
   const long long want = std::max((n + 4 * CV_RESIDENT_NT - 1) / (4 * CV_RESIDENT_NT), 1ll);
-  if (want <= 8) {  // one cluster of the portable size
+  // one cluster of the portable size; a context with part of the SMs may not
+  // have as many next to each other
+  if (want <= 8 && sms == device) {
     int c = 1;
     while (c < want) c *= 2;
     return {c, true, true};

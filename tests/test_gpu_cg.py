@@ -1,5 +1,7 @@
 """Mixed-precision CG: FP32/BF16 inner solves, FP64 residual and update.
 The final residual is recomputed on the host by the oracle's FP64 SpMV."""
+import contextlib
+import ctypes
 import time
 
 import numpy as np
@@ -150,6 +152,52 @@ def test_grid_barriers_that_run_out_end_the_solve(n, graph):
     xd.zero_()
     assert smat.cg_mixed(A64, A32, bd, xd, **opts)["converged"]
     assert torch.equal(xd, good)              # the context is usable, the solve reproducible
+    A64.close(), A32.close()
+
+
+@contextlib.contextmanager
+def part_of_the_sms(count):
+    """A green context of about `count` SMs, current inside the block."""
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def call(name, *args):
+        st = getattr(cu, name)(*args)
+        assert st == 0, (name, st)
+
+    torch.cuda.current_stream().synchronize()
+    dev, groups = ctypes.c_int(), ctypes.c_uint(1)
+    whole, part, rest = (ctypes.create_string_buffer(512) for _ in range(3))   # CUdevResource
+    desc, green, ctx, old = (ctypes.c_void_p() for _ in range(4))
+    call("cuDeviceGet", ctypes.byref(dev), 0)
+    call("cuDeviceGetDevResource", dev, whole, 1)                              # CU_DEV_RESOURCE_TYPE_SM
+    call("cuDevSmResourceSplitByCount", part, ctypes.byref(groups), whole, rest, 0, count)
+    call("cuDevResourceGenerateDesc", ctypes.byref(desc), part, 1)
+    call("cuGreenCtxCreate", ctypes.byref(green), desc, dev, 1)                # CU_GREEN_CTX_DEFAULT_STREAM
+    call("cuCtxFromGreenCtx", ctypes.byref(ctx), green)
+    call("cuCtxPushCurrent_v2", ctx)
+    try:
+        yield
+    finally:
+        call("cuCtxSynchronize")
+        call("cuCtxPopCurrent_v2", ctypes.byref(old))
+        call("cuGreenCtxDestroy", green)
+
+
+@pytest.mark.parametrize("n", [20000, 40000, 1400001])
+def test_context_with_part_of_the_sms(n):
+    # the vector kernel waits for all of its CTAs: no more than the context's
+    # SMs hold at once
+    A = tridiagonal(n)
+    x_true = synth.uniform(3, 5, n)
+    b = oracle.spmv_csr(n, A.rowptr, A.colidx, A.val, x_true, threads=8)
+    A64, A32 = handles(A, tune=False)
+    bd = torch.from_numpy(b).to(DEV)
+    xd = torch.zeros(n, dtype=torch.float64, device=DEV)
+    with part_of_the_sms(16):
+        info = smat.cg_mixed(A64, A32, bd, xd, stream=0, rtol=1e-12)
+    assert info["converged"], info
+    err = np.linalg.norm(xd.cpu().numpy() - x_true) / np.linalg.norm(x_true)
+    assert err <= 4e-12, err
     A64.close(), A32.close()
 
 
