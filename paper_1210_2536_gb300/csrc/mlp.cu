@@ -20,6 +20,7 @@
 // mlp_forward of one sample 25.8 -> 5.4 us; a training step 53 -> 35 us, now the
 // host's time to issue its launches.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "smat_internal.h"
@@ -273,12 +274,17 @@ __global__ void __launch_bounds__(128) adam_kernel(float *__restrict__ p, const 
   }
 }
 
-cudaError_t set_smem(const void *fn) {
-  static bool done[2] = {false, false};
-  int k = fn == (const void *)mlp_forward_kernel ? 0 : 1;
-  if (done[k]) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(STOT * sizeof(float)));
-  if (e == cudaSuccess) done[k] = true;
+static_assert(SFWD * sizeof(float) <= 48 * 1024, "the forward kernel needs no larger shared memory limit");
+
+// mlp_loss_grad_kernel's shared memory is above the default limit, which is
+// raised per device.
+cudaError_t raise_smem_limit() {
+  static std::atomic<bool> raised[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev < 64 && raised[dev].load())) return e;
+  e = cudaFuncSetAttribute(mlp_loss_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(STOT * sizeof(float)));
+  if (e == cudaSuccess && dev < 64) raised[dev] = true;
   return e;
 }
 
@@ -286,8 +292,6 @@ cudaError_t set_smem(const void *fn) {
 
 cudaError_t launch_mlp_forward(const float *params, const float *X, int B, float *logits, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
-  cudaError_t e = set_smem((const void *)mlp_forward_kernel);
-  if (e != cudaSuccess) return e;
   return launch_pdl(mlp_forward_kernel, dim3((B + S - 1) / S), dim3(NT), SFWD * sizeof(float), s, params, X, (int)B,
                     logits);
 }
@@ -309,7 +313,7 @@ smat_status_t smat_mlp_loss_grad(const float *params, const float *X, const floa
                                  float *loss, float *work, void *stream) {
   if (B <= 0 || !params || !X || !T || !grad || !loss || !work) return SMAT_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  if (set_smem((const void *)mlp_loss_grad_kernel) != cudaSuccess) return SMAT_ERR_CUDA;
+  if (raise_smem_limit() != cudaSuccess) return SMAT_ERR_CUDA;
   int nblk = (B + S - 1) / S;
   cudaError_t e = launch_pdl(mlp_loss_grad_kernel, dim3(nblk), dim3(NT), STOT * sizeof(float), s, params, X, T, (int)B,
                              work);

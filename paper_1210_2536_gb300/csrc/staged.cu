@@ -201,19 +201,23 @@ template <typename V, int MODE, int CFG>
 cudaError_t dia_staged_cfg(const smat_s *h, const StagedGeom &g, typename Compute<V>::T alpha, const void *x,
                            typename Compute<V>::T beta, void *y, cudaStream_t s, long long wait_limit) {
   typedef typename Compute<V>::T T;
-  static size_t dyn_max = 0;  // per process; the attribute is per function
+  static std::atomic<size_t> raised[64] = {};  // the attribute is per function and device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  size_t dyn_max = dev < 64 ? raised[dev].load() : 0;
   if (dyn_max == 0) {
     // dynamic plus static shared memory may not exceed the opt-in limit
-    int dev = 0, optin = 0;
+    int optin = 0;
     cudaFuncAttributes fa;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, dia_staged_kernel<V, MODE, CFG>);
     if (e != cudaSuccess) return e;
     const size_t lim = (size_t)optin - fa.sharedSizeBytes;
     e = cudaFuncSetAttribute(dia_staged_kernel<V, MODE, CFG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
     if (e != cudaSuccess) return e;
     dyn_max = lim;
+    if (dev < 64) raised[dev] = lim;
   }
   if (g.smem > dyn_max) return cudaErrorNotSupported;
   (void)launch_pdl(dia_staged_kernel<V, MODE, CFG>, dim3(g.grid), dim3(32 * (ST_CFG[CFG].warps + 1)), g.smem, s,
