@@ -907,6 +907,10 @@ smat_status_t prepare_variant(smat_s *h, int v, cudaStream_t s) {
   TRYS(build_format(h, fmt, s));
   TRYS(ensure_scratch(h, v));
   if (v == SMAT_V_CSR_MERGE && !h->flat_row && h->m > 0) {
+    // not on a stream that is capturing, which cannot be read back from
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    TRY(cudaStreamIsCapturing(s, &cs));
+    if (cs != cudaStreamCaptureStatusNone) s = dev_pool().s;
     void *p = nullptr;
     DevBuf gaps(s);
     int found = 0;

@@ -117,6 +117,25 @@ def test_every_row_takes_beta_once(name, A, dtype):
     M.close(), N.close()
 
 
+@pytest.mark.parametrize("name", ["gaps_past_the_warp_s_own", "ragged_mix"])
+def test_first_product_while_capturing(name):
+    # a relaxed capture may hold a handle's first CSR_MERGE product: what the
+    # kernel needs to know of the rows is found beside the capture
+    A = dict(_cases())[name]
+    M = smat.SpMatrix(A.m, A.n, A.rowptr, A.colidx, A.val, "f64")
+    x, y0 = synth.uniform(1, 1, A.n), synth.uniform(2, 1, A.m)
+    xd, y = (torch.from_numpy(t).to(DEV) for t in (x, y0.copy()))
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+        M.spmv(xd, y, 2.0, -0.5, variant=smat.SMAT_V_CSR_MERGE, stream=s)
+    g.replay()
+    torch.cuda.synchronize()
+    ref, scale = reference(A, A.val, x, 2.0, -0.5, y0)
+    assert_close_rows(y.cpu().numpy(), ref, scale, TOL["f64"], name)
+    M.close()
+
+
 def test_noalloc_several_chunks_per_tile():
     # 65536 tiles of one chunk hold 16.8 M entries: this matrix takes two per
     # tile, with rows that cross chunks and tiles
