@@ -291,9 +291,11 @@ smat_status_t smat_get_kernel(smat_handle_t h, smat_variant_t v, int32_t *kernel
 smat_status_t smat_spmv_host(smat_handle_t h, const void *alpha, const void *x_host,
                              const void *beta, void *y_host, void *stream);
 
-/* Matrix bytes one product through variant v reads (the format's arrays; x
- * and y, common to every variant, excluded): the quantity the execute-and-
- * measure search breaks near-ties on.  Computes the features first if
+/* Matrix bytes of one product through variant v: the format's arrays as it
+ * defines them (x and y, common to every variant, excluded), the quantity the
+ * execute-and-measure search breaks near-ties on.  COO's entries, HYB's tail
+ * and SPLIT's short rows count with a 4-byte row index each; the kernels read
+ * about one bit per entry in its place.  Computes the features first if
  * needed; SMAT_ERR_UNSUPPORTED for HYB / SELL / BCSR / SPLIT before their
  * layout has been measured (by smat_tune or smat_convert). */
 smat_status_t smat_variant_bytes(smat_handle_t h, smat_variant_t v, double *bytes);

@@ -624,7 +624,7 @@ class SpMatrix:
         return y
 
     def variant_bytes(self, variant) -> float:
-        """Matrix bytes one product through `variant` reads (smat_variant_bytes)."""
+        """Matrix bytes of `variant`'s format, row index per listed entry included (smat_variant_bytes)."""
         b = ctypes.c_double()
         _check(lib().smat_variant_bytes(self.h, int(variant), ctypes.byref(b)), "smat_variant_bytes")
         return b.value

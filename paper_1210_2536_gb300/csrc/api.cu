@@ -223,7 +223,10 @@ double csr_bytes(const smat_s *h) { return (double)(h->esz + 4) * h->nnz + 4.0 *
 double ell_bytes(const smat_s *h) { return (double)(h->esz + 4) * h->f.max_rd * h->P; }
 double dia_bytes(const smat_s *h) { return (double)h->esz * h->f.ndiags * h->P + 4.0 * h->f.ndiags; }
 
-// Matrix bytes one product through `v` reads (x and y are common to all).
+// Matrix bytes of a product through `v` as its format defines the arrays (x and
+// y are common to all).  COO's entries, HYB's tail and SPLIT's short rows count
+// a 4-byte row index each, which the kernels read as row ends (about one bit
+// per entry): these counts also decide what is admissible under bytes_cap.
 double variant_bytes(const smat_s *h, int v) {
   switch (v) {
     case SMAT_V_ELL: return ell_bytes(h);

@@ -348,8 +348,9 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
   // the members' order, a branch of several large products outlived the rest,
   // and every member's own launches (mode 2) lost to the persistent kernels
   // beside the others' launches.  us per product, before and now: 29 FP64
-  // matrices on the 128^3 hierarchy 284 -> 267, 27 on 50^3 159 -> 148, 16 FP32
-  // on 96^3 57 -> 55; six branches 270, 152 and 57, sixteen as eight.
+  // matrices on the 128^3 hierarchy 281 -> 271 (two tunings of one batch differ
+  // by 2 %), 27 on 50^3 159 -> 148, 16 FP32 on 96^3 57 -> 55; six branches and
+  // sixteen were no faster than eight on any of the three.
   std::vector<size_t> own_order;
   for (size_t i = 0; i < n; ++i)
     if (b->own[i]) own_order.push_back(i);
@@ -452,7 +453,8 @@ smat_status_t smat_batch_create(smat_batch_t *out, const smat_handle_t *hs, int3
   auto fail = [&](smat_status_t s) { smat_batch_destroy(b); return s; };
   // the persistent kernels go ahead of the members' own launches, whose many
   // short CTAs would otherwise hold the SMs first: they run longest (29 FP64
-  // matrices on the 128^3 hierarchy 285 -> 281 us)
+  // matrices on the 128^3 hierarchy 285 -> 281 us, and 277 to 278 in another
+  // run: within the 2 % by which two tunings of one batch differ)
   int low = 0, high = 0;
   cudaError_t e = cudaDeviceGetStreamPriorityRange(&low, &high);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->cap, cudaStreamNonBlocking, high);

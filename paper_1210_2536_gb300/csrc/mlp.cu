@@ -17,8 +17,8 @@
 // and a thread computes one output of four samples (or eight rows of one
 // column of a weight gradient), so that 16 multiply-adds share five loads.
 // mlp_loss_grad at 128 samples: 43.3 us before, 13.3 us now (ncu, cold caches);
-// mlp_forward of one sample 25.8 -> 5.4 us; a training step 53 -> 35 us, now the
-// host's time to issue its launches.
+// mlp_forward of one sample 25.8 -> 5.4 us; a training step 53 -> 35 to 41 us, now
+// the host's time to issue its launches.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
