@@ -39,6 +39,10 @@
  * with other calls on the handle.  The selector model and the plan cache are
  * process-wide and guarded: smat_load_model / smat_set_model may run while
  * other threads tune (a tuning predicts from a copy of the model).
+ * smat_cg_mixed (with use_graph) and the batch calls that build a graph capture
+ * it on streams of their own.  CUDA refuses to wait for the whole device during
+ * a capture; the library's own such waits (freeing device memory) let captures
+ * finish first, a caller's cudaDeviceSynchronize on another thread does not.
  */
 #ifndef SMAT_H
 #define SMAT_H

@@ -90,6 +90,16 @@ DevPool &dev_pool() {
   return d;
 }
 
+std::shared_mutex &capture_mu() {
+  static std::shared_mutex mu;
+  return mu;
+}
+
+static cudaError_t wait_for_device() {
+  std::unique_lock<std::shared_mutex> lk(capture_mu());
+  return cudaDeviceSynchronize();
+}
+
 // Long-lived buffers (formats, handle copies): ready for every stream when
 // this returns.
 cudaError_t dev_alloc(void **p, size_t bytes) {
@@ -116,7 +126,7 @@ void dev_free(void *p) {
     cudaFree(p);
     return;
   }
-  cudaDeviceSynchronize();
+  wait_for_device();
   cudaFreeAsync(p, d.s);
 }
 
@@ -822,6 +832,11 @@ smat_status_t build_format(smat_s *h, int fmt, cudaStream_t s) {
 }  // namespace
 
 cudaError_t stream_scratch(const smat_s *h, cudaStream_t s, Scratch *out, bool claim) {
+  // freed once scratch_mu is given back: a capture takes it, and dev_free waits for captures
+  struct Later {
+    void *p = nullptr;
+    ~Later() { dev_free(p); }
+  } later;
   std::lock_guard<std::mutex> lock(h->scratch_mu);
   if (!claim) {
     *out = Scratch{h->carry, h->split_part};
@@ -847,7 +862,7 @@ cudaError_t stream_scratch(const smat_s *h, cudaStream_t s, Scratch *out, bool c
     if (e != cudaSuccess) return e;
     if (hit) {
       cudaStreamSynchronize(s);  // the old buffer's products on s are done
-      dev_free(hit->p);
+      later.p = hit->p;
       hit->p = p;
       hit->bytes = need;
     } else {
@@ -860,14 +875,18 @@ cudaError_t stream_scratch(const smat_s *h, cudaStream_t s, Scratch *out, bool c
 }
 
 void release_stream_scratch(const smat_s *h, cudaStream_t s) {
-  std::lock_guard<std::mutex> lock(h->scratch_mu);
-  if (h->scratch_owned && h->scratch_owner == s) h->scratch_owned = false;
-  for (size_t i = 0; i < h->more_scratch.size(); ++i)
-    if (h->more_scratch[i].stream == s) {
-      dev_free(h->more_scratch[i].p);
-      h->more_scratch.erase(h->more_scratch.begin() + (long)i);
-      break;
-    }
+  void *own = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(h->scratch_mu);
+    if (h->scratch_owned && h->scratch_owner == s) h->scratch_owned = false;
+    for (size_t i = 0; i < h->more_scratch.size(); ++i)
+      if (h->more_scratch[i].stream == s) {
+        own = h->more_scratch[i].p;
+        h->more_scratch.erase(h->more_scratch.begin() + (long)i);
+        break;
+      }
+  }
+  dev_free(own);
 }
 
 void free_stream_scratch(smat_s *h) {
@@ -1200,7 +1219,7 @@ smat_status_t smat_release_cached_memory(void) {
     DevPool &d = pools()[dev];
     if (!d.pool) continue;
     ok = cudaSetDevice(dev) == cudaSuccess && ok;
-    ok = cudaDeviceSynchronize() == cudaSuccess && ok;
+    ok = wait_for_device() == cudaSuccess && ok;
     ok = cudaMemPoolTrimTo(d.pool, 0) == cudaSuccess && ok;
   }
   cudaSetDevice(cur);

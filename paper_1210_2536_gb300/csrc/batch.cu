@@ -400,6 +400,7 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
   b->ctas_per_sm = ctas_per_sm;
   // capture: reset the tile counters, then one persistent kernel per format
   // kind on parallel branches of the graph
+  std::shared_lock<std::shared_mutex> capturing(capture_mu());
   BTRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
   cudaError_t err = cudaMemsetAsync(b->d_counter, 0, NKIND * sizeof(unsigned int), b->cap);
   if (err == cudaSuccess) err = cudaEventRecord(b->ev_fork, b->cap);
@@ -425,6 +426,7 @@ smat_status_t build_plan(smat_batch_s *b, int scale, int ctas_per_sm, int own_mo
     }
   }
   cudaError_t e3 = cudaStreamEndCapture(b->cap, &b->graph);
+  capturing.unlock();
   BTRY(err);
   BTRY(e3);
   BTRY(cudaGraphInstantiate(&b->exec, b->graph, 0));

@@ -580,10 +580,12 @@ extern "C" smat_status_t smat_cg_mixed(smat_handle_t a64, smat_handle_t a32, con
         if (o.max_total_inner > 0) k = std::min(k, o.max_total_inner - inf.inner_total - it);
         if (o.use_graph && k == chunk) {
           if (!gexec) {  // capture one chunk of iterations once, replay it afterwards
+            std::shared_lock<std::shared_mutex> capturing(capture_mu());
             if (!chk(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal))) { ok = false; break; }
             bool cap_ok = true;
             for (int j = 0; j < chunk && cap_ok; ++j) cap_ok = inner_iteration();
             cudaError_t ce = cudaStreamEndCapture(s, &graph);
+            capturing.unlock();
             if (!cap_ok || !chk(ce)) { ok = false; break; }
             if (!chk(cudaGraphInstantiate(&gexec, graph, 0))) { ok = false; break; }
           }

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <shared_mutex>
 #include <vector>
 
 #include "smat.h"
@@ -23,6 +24,11 @@ void dev_free(void *p);
 // Temporaries used on one stream only, allocated and freed in its order.
 cudaError_t tmp_alloc(void **p, size_t bytes, cudaStream_t s);
 void tmp_free(void *p, cudaStream_t s);
+
+// Held shared while a thread captures a graph, and alone while one waits for the
+// whole device: CUDA refuses that wait while any stream captures, and the
+// capture is lost too.  Nothing that a capture takes is held while waiting.
+std::shared_mutex &capture_mu();
 
 // Plan cache (plan_cache.cu): the structural key, computed once per handle,
 // and the process-wide table of plans.

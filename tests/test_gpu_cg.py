@@ -2,6 +2,7 @@
 The final residual is recomputed on the host by the oracle's FP64 SpMV."""
 import contextlib
 import ctypes
+import threading
 import time
 
 import numpy as np
@@ -199,6 +200,39 @@ def test_context_with_part_of_the_sms(n):
     err = np.linalg.norm(xd.cpu().numpy() - x_true) / np.linalg.norm(x_true)
     assert err <= 4e-12, err
     A64.close(), A32.close()
+
+
+def test_solves_on_several_threads():
+    # each solve captures its iterations and frees its workspace, which waits
+    # for the device: CUDA allows no such wait while another thread captures
+    n, reps = 60000, 10
+    A = tridiagonal(n)
+    b = oracle.spmv_csr(n, A.rowptr, A.colidx, A.val, synth.uniform(3, 5, n), threads=8)
+    bd = torch.from_numpy(b).to(DEV)
+    pairs = [handles(A, tune=False) for _ in range(4)]
+    xs = [[torch.zeros(n, dtype=torch.float64, device=DEV) for _ in range(reps)] for _ in pairs]
+    first = torch.zeros(n, dtype=torch.float64, device=DEV)
+    assert smat.cg_mixed(*pairs[0], bd, first, stream=0, rtol=1e-12)["converged"]
+    torch.cuda.synchronize()
+    status = [[] for _ in pairs]
+
+    def work(k):
+        for x in xs[k]:
+            st, info = smat.smat_cg_mixed(pairs[k][0].h, pairs[k][1].h, bd.data_ptr(), x.data_ptr(), opts, 0)
+            status[k].append(st)
+
+    opts = smat.smat_cg_opts_default()
+    opts.rtol = 1e-12
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(pairs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert status == [[smat.SMAT_OK] * reps] * len(pairs), status
+    assert all(torch.equal(x, first) for row in xs for x in row)
+    for A64, A32 in pairs:
+        A64.close(), A32.close()
 
 
 def arrow(n):
